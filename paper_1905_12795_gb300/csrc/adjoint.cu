@@ -22,9 +22,9 @@
 // forward field the adjoint pass needs (its gradient term then costs one
 // pointwise read per point-step instead of a staged tile and a second
 // Laplacian), and leaves its traces for adj_residual_kernel;
-// adj_fwd_kernel is the per-step form for grids neither can hold (and order
-// 16), which keeps its time levels in two adjoint slots and writes the
-// same history.  The per-step kernels here run over all instances at once
+// at order 16 on the plain streaming kernel; adj_fwd_kernel is the per-step
+// form for grids none of them can hold, which keeps its time levels in two
+// adjoint slots and writes the same history.  The per-step kernels here run over all instances at once
 // (blockIdx.y = instance), one launch per time step (the time loops replay as
 // one CUDA graph).  They stage the fields their Laplacians read in
 // shared-memory tiles and give each thread a few rows of one float4 group.
@@ -90,7 +90,6 @@ __global__ void adj_prep_kernel(GridDev g, const float *a, float *B)
 // TZ = 4 when that still gives every SM enough blocks (less halo re-read, one
 // wave), else 2 or 1 (more, smaller blocks to fill the GPU).
 constexpr int TW = 16, TILE_THREADS = TW * 8;
-constexpr int FWD_TZ8 = 4;   // forward rows per thread at radius 8 when the tiles fill the GPU
 
 template <int R> struct Tile {
     static constexpr int XG = (R + 3) / 4;     // halo groups each side
@@ -646,9 +645,8 @@ int tile_count(const GridDev &g, int TT) { return tiles_x(g) * ((g.NZ + TT - 1) 
 using StepFn = void (*)(GridDev, const AdjInst *, int);
 using Step1Fn = void (*)(GridDev, const AdjInst *, int, int);
 
-StepFn fwd_fn(int R, int TZ)
+StepFn fwd_fn(int R)
 {
-    if (R == 8) return TZ == 4 ? adj_fwd_kernel<8, 4> : (TZ == 2 ? adj_fwd_kernel<8, 2> : adj_fwd_kernel<8, 1>);
     if (R == 4) return adj_fwd_kernel<4, 1>;
     return R == 2 ? adj_fwd_kernel<2, 1> : adj_fwd_kernel<1, 1>;
 }
@@ -681,20 +679,6 @@ int adj_rows_per_thread(const GridDev &g, int n_inst)
     return 1;
 }
 
-// rows per thread of the forward step: 1, except at radius 8, where a tile
-// of 8 rows stages 3 times its rows (2R = 16 halo rows): there 4 rows (1.5
-// times) while that gives every SM 7 tile blocks, else 2 while that gives 3
-int adj_fwd_rows_per_thread(const GridDev &g, int n_inst)
-{
-    if (g.R < 8) return 1;
-    int sms = 0, dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        sms = 1;
-    if ((long long)tile_count(g, 32) * n_inst >= 7LL * sms) return FWD_TZ8;
-    if ((long long)tile_count(g, 16) * n_inst >= 3LL * sms) return 2;
-    return 1;
-}
-
 }  // namespace
 
 cudaError_t launch_adj_prep(const GridDev &g, const float *a, float *B, int M, cudaStream_t st)
@@ -708,9 +692,8 @@ cudaError_t launch_adj_forward(const GridDev &g, const AdjInst *insts, int n_ins
 {
     // step n also records e_{n-1} (in an extra block); the last record
     // follows the loop
-    const int tz = adj_fwd_rows_per_thread(g, n_inst);
-    const dim3 grid(tile_count(g, 8 * tz) + 1, n_inst);
-    const StepFn fn = fwd_fn(g.R, tz);
+    const dim3 grid(tile_count(g, 8) + 1, n_inst);
+    const StepFn fn = fwd_fn(g.R);
     for (int n = 0; n < g.nt; ++n) fn<<<grid, TILE_THREADS, 0, st>>>(g, insts, n);
     adj_record_kernel<<<n_inst, rec_threads, 0, st>>>(g, insts, g.nt - 1);
     return cudaGetLastError();

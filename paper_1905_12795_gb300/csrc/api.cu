@@ -98,11 +98,11 @@ struct empso_ctx {
     size_t stage_cap = 0;        // bytes
     cudaEvent_t stage_free = nullptr;
     int *counter = nullptr;
+    unsigned char *wave_ws = nullptr;     // plain streaming kernel: queue, group barriers, partial sums
+    size_t wave_ws_cap = 0;               // bytes
 
     // launch shape of the modelling kernel
     int kernel_kind = EMPSO_KERNEL_AUTO;
-    int wave_threads = 512;
-    int wave_ctas_per_sm = 1;
     size_t smem_optin = 0;          // max dynamic shared memory per block
     int forced_C = 0;               // 0: choose the cluster size, else use this one
     int forced_rows = 0;            // on-chip kernel: 0 choose the rows per thread, else use this many
@@ -186,8 +186,10 @@ struct empso_ctx {
         size_t rtab_cap = 0;
         int *counter = nullptr;          // its work queue
         size_t counter_cap = 0;
-        float4 *slots = nullptr;         // L2 cluster forward pass: two time levels per cluster
-        size_t slots_cap = 0;
+        float4 *slots = nullptr;         // L2 cluster and plain streaming forward pass: two time levels per
+        size_t slots_cap = 0;            // instance in flight
+        unsigned char *wave_ws = nullptr;   // plain streaming forward pass
+        size_t wave_ws_cap = 0;
         // forward + adjoint time loops captured once per grid, instance count
         // and instance table (their kernels read everything else from it)
         std::vector<std::pair<std::string, cudaGraphExec_t>> graphs;
@@ -445,6 +447,8 @@ struct Plan {
     int l2C = 0, l2_clusters = 0, l2_threads = 0;
     long long l2_slot_f4 = 0;
     size_t l2_smem = 0;
+    WaveSplit wave{};                  // plain streaming kernel: instances in flight, CTAs for each
+    int wave_R = 0;                    // its stencil radius (0: the grids differ)
     bool stream_tma = false;           // streaming path: row-pipelined bulk-copy kernel
     int st_threads = 0, st_R = 0, rec_max = 0;
     size_t st_smem = 0;
@@ -625,7 +629,7 @@ empso_status plan_batch(empso_ctx *ctx, const Models &mod, const empso_shot *sho
     }
     if (kind == EMPSO_KERNEL_CLUSTER_L2 && !p.l2)
         return fail(ctx, EMPSO_UNSUPPORTED, "the batch does not fit the L2 cluster kernel");
-    int max_ctas = ctx->sm_count * ctx->wave_ctas_per_sm;
+    int max_ctas = 0;
     if (!p.resident && !p.l2 && resR > 0) {
         // row-pipelined streaming kernel: one thread per float4 column group
         int nq = 0, pitch = 0, nrec_max = 0;
@@ -646,6 +650,22 @@ empso_status plan_batch(empso_ctx *ctx, const Models &mod, const empso_shot *sho
             const int per_sm = std::max(1, (int)(ctx->smem_optin / std::max<size_t>(sm, 1)));
             max_ctas = ctx->sm_count * std::min(per_sm, 2);
         }
+    }
+    if (!p.resident && !p.l2 && !p.stream_tma) {
+        std::vector<const GridDev *> used;
+        long long inst_bytes = 1;
+        for (int gid = 0; gid < ng; ++gid) {
+            if (p.fbase[gid] < 0) continue;
+            const GridDev &g = ctx->grids[gid].dev;
+            used.push_back(&g);
+            p.wave_R = used.size() == 1 || p.wave_R == g.R ? g.R : 0;
+            inst_bytes = std::max(inst_bytes, 12 * g.field);
+        }
+        p.wave = wave_split(used.data(), (int)used.size(), p.wave_R, p.n_inst, L2_BUDGET_BYTES / inst_bytes);
+        if (p.wave.group < 1) return fail(ctx, EMPSO_CUDA_ERROR, "occupancy of the streaming kernel");
+        // sized once, for any split of this device (captured generations keep the pointer)
+        if ((rc = grow(ctx, (void **)&ctx->wave_ws, &ctx->wave_ws_cap, wave_ws_bytes(), 1)) != EMPSO_OK) return rc;
+        max_ctas = p.wave.flight;
     }
     p.n_ctas = (int)std::min<long long>(p.n_inst, max_ctas);
     if ((rc = grow(ctx, (void **)&ctx->fields, &ctx->fields_cap, sizeof(float) * ftotal,
@@ -790,11 +810,11 @@ empso_status enqueue_batch(empso_ctx *ctx, const Models &mod, const Plan &p, dou
         ctx->last_C = 1;
         ctx->last_groups = p.n_ctas;
     } else {
-        CK(ctx, launch_wave(ctx->grids_dev, p.insts, (int)p.n_inst, ctx->counter, ctx->slots,
-                            2 * p.maxfield, p.n_ctas, ctx->wave_threads, ctx->partial, st));
+        CK(ctx, launch_wave(p.wave_R, ctx->grids_dev, p.insts, (int)p.n_inst, p.wave, ctx->wave_ws, ctx->slots,
+                            2 * p.maxfield, ctx->dev_err, ctx->partial, st));
         ctx->last_path = 1;
         ctx->last_C = 1;
-        ctx->last_groups = p.n_ctas;
+        ctx->last_groups = p.wave.flight * p.wave.group;
     }
     if (ctx->timing) CK(ctx, mark(ctx->tev[2], st));
     if (misfit)
@@ -878,6 +898,7 @@ void free_ctx(empso_ctx *c)
     cudaFree(c->partial);
     cudaFree(c->stage_dev);
     cudaFree(c->counter);
+    cudaFree(c->wave_ws);
     cudaFree(c->dev_err);
     cudaFree(c->nonfinite);
     cudaFree(c->adj.a);       // B lies inside a; G and J inside mu
@@ -893,6 +914,7 @@ void free_ctx(empso_ctx *c)
     cudaFree(c->adj.rtab);
     cudaFree(c->adj.counter);
     cudaFree(c->adj.slots);
+    cudaFree(c->adj.wave_ws);
     cudaFree(c->pso_mem);
     cudaFree(c->pso_int);
     cudaFree(c->xf);
@@ -997,7 +1019,6 @@ empso_status empso_create(const empso_grid *grids, int32_t ngrids, const float *
     if ((rc = ck(cudaMalloc(&ctx->counter, sizeof(int)), "counter")) ||
         (rc = ck(cudaEventCreateWithFlags(&ctx->stage_free, cudaEventDisableTiming), "event")))
         return bail(rc);
-    ctx->wave_ctas_per_sm = std::max(1, wave_max_ctas_per_sm(ctx->wave_threads));
     {
         int optin = 0;
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device);
@@ -1322,8 +1343,18 @@ empso_status gradient_impl(empso_ctx *ctx, const float *vel, int M, const empso_
     }
     if (ctx->kernel_kind == EMPSO_KERNEL_CLUSTER_L2 && !lC)
         return fail(ctx, EMPSO_UNSUPPORTED, "gradient: the grid does not fit the L2 cluster kernel");
+    // the cluster kernels hold stencils up to radius 4; order 16 runs its forward
+    // pass on the plain streaming kernel, which streams the history out too
+    WaveSplit split{};
+    if (g.R > MAX_R_FAST) {
+        const GridDev *gp = &g;
+        split = wave_split(&gp, 1, g.R, I, L2_BUDGET_BYTES / (12 * g.field), true);
+        if (split.group < 1) return fail(ctx, EMPSO_CUDA_ERROR, "gradient: occupancy of the streaming kernel");
+        if ((rc = adj_grow(ctx, &W.wave_ws, &W.wave_ws_cap, wave_ws_bytes(), nullptr))) return rc;
+        if ((rc = adj_grow(ctx, &W.slots, &W.slots_cap, F / 2 * split.flight, nullptr))) return rc;
+    }
     const size_t r_ofs = ((size_t)I * sizeof(Inst) + 255) / 256 * 256;
-    const bool table = rC || lC;
+    const bool table = rC || lC || split.group;
     if (table) {
         if ((rc = adj_grow(ctx, &W.rtab, &W.rtab_cap, r_ofs + sizeof(int4) * (size_t)I, nullptr))) return rc;
         if ((rc = adj_grow(ctx, &W.counter, &W.counter_cap, 1, nullptr))) return rc;
@@ -1407,6 +1438,11 @@ empso_status gradient_impl(empso_ctx *ctx, const float *vel, int M, const empso_
                 ce = launch_wave_l2(g.R, ctx->grids_dev, reinterpret_cast<const Inst *>(W.rtab), (int)I, W.counter,
                                     lC, l_nc, l_threads, W.slots, l_slot, rec_max, l_smem, W.phi,
                                     ctx->cap_stream, true);
+            if (ce == cudaSuccess) ce = launch_adj_residual(g, W.insts, (int)I, rec_max, ctx->cap_stream);
+        } else if (split.group) {
+            ce = launch_wave(g.R, ctx->grids_dev, reinterpret_cast<const Inst *>(W.rtab), (int)I, split, W.wave_ws,
+                             reinterpret_cast<float *>(W.slots), 2 * g.field, ctx->dev_err, W.phi, ctx->cap_stream,
+                             !forward_only);
             if (ce == cudaSuccess) ce = launch_adj_residual(g, W.insts, (int)I, rec_max, ctx->cap_stream);
         } else {
             // the per-step forward pass with its time levels in the (zeroed)

@@ -168,12 +168,23 @@ cudaError_t launch_interp(const GridDev &g, const float *particles, int P, float
                           long long field_stride, float *vel_out, cudaStream_t st);
 cudaError_t launch_vel_to_field(const GridDev &g, const float *vel, int M, float *a_fields,
                                 long long field_stride, cudaStream_t st);
-cudaError_t launch_wave(const GridDev *grids_dev, const Inst *insts, int n_inst,
-                        int *counter, float *slots, long long slot_floats, int n_ctas,
-                        int threads, double *partial, cudaStream_t st);
+// Plain streaming variant (wave.cu): `flight` instances at once on `group`
+// co-resident CTAs each.  R: the stencil radius of every grid, 0 when they
+// differ.  ws: wave_ws_bytes() (enough for any split; the launch clears what it
+// uses).  hist (radius 8 only): also L u^n of every step into Inst::hist, slot n + 1.
+constexpr int WAVE_MAX_CTAS = 4096;      // co-resident CTAs of any device
+struct WaveSplit {
+    int flight, group;
+};
+int wave_max_ctas(int R, bool hist = false);
+WaveSplit wave_split(const GridDev *const *grids, int n_grids, int R, long long n_inst, long long by_l2,
+                     bool hist = false);
+constexpr size_t wave_ws_bytes(int flight = WAVE_MAX_CTAS) { return 128 * (1 + (size_t)flight) + sizeof(double) * WAVE_MAX_CTAS; }
+cudaError_t launch_wave(int R, const GridDev *grids_dev, const Inst *insts, int n_inst, const WaveSplit &s,
+                        void *ws, float *slots, long long slot_floats, int *err, double *partial,
+                        cudaStream_t st, bool hist = false);
 cudaError_t launch_finalize(const double *partial, const float *weights, int P, int S,
                             double *misfit, unsigned long long *nf, cudaStream_t st);
-int wave_max_ctas_per_sm(int threads);
 
 // On-chip variant (wave_resident.cu): one thread-block cluster per instance.
 // float4 per slab row of its damping table: one for the column groups outside

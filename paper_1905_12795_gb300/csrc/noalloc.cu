@@ -28,8 +28,13 @@ constexpr int NOALLOC_MAX_DEVICES = 64;
 // cudaGetSymbolAddress.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_SCRATCH_BYTES];
 
+// The modelling launch's workspace, for at most this many instances at once.
+constexpr int NOALLOC_FLIGHT = 64;
+static __device__ __align__(256) unsigned char g_noalloc_ws[wave_ws_bytes(NOALLOC_FLIGHT)];
+
 std::mutex g_mu;
 void *g_scratch_addr[NOALLOC_MAX_DEVICES] = {};
+void *g_ws_addr[NOALLOC_MAX_DEVICES] = {};
 
 struct SetupParams {
     GridDev g;
@@ -47,7 +52,7 @@ struct Layout {
     float *weights;
     Inst *insts;
     double *partial;
-    int *counter;
+    int *err;                  // status word of the launch's bounded waits
     float *fields;
     float *slots;
     size_t used;
@@ -75,7 +80,7 @@ Layout carve(unsigned char *base, const GridDev &g, int S, int nrec_total, int M
     L.weights = reinterpret_cast<float *>(take(sizeof(float) * S));
     L.insts = reinterpret_cast<Inst *>(take(sizeof(Inst) * (size_t)M * S));
     L.partial = reinterpret_cast<double *>(take(sizeof(double) * (size_t)M * S));
-    L.counter = reinterpret_cast<int *>(take(sizeof(int)));
+    L.err = reinterpret_cast<int *>(take(sizeof(int)));
     L.fields = reinterpret_cast<float *>(take(sizeof(float) * (size_t)M * g.field));
     L.slots = reinterpret_cast<float *>(take(sizeof(float) * 2 * (size_t)g.field * n_slots));
     L.used = o;
@@ -165,6 +170,7 @@ extern "C" empso_status eval_models_noalloc(const empso_grid *grid, const float 
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= NOALLOC_MAX_DEVICES)
         return nfail(EMPSO_CUDA_ERROR, "no current CUDA device");
     unsigned char *base;
+    void *ws;
     {
         std::lock_guard<std::mutex> lock(g_mu);
         if (!g_scratch_addr[dev]) {
@@ -173,9 +179,15 @@ extern "C" empso_status eval_models_noalloc(const empso_grid *grid, const float 
             if (e != cudaSuccess || !ptr)
                 return nfail(EMPSO_CUDA_ERROR, std::string("cudaGetSymbolAddress: ") +
                                                    cudaGetErrorString(e));
+            void *wptr = nullptr;
+            e = cudaGetSymbolAddress(&wptr, g_noalloc_ws);
+            if (e != cudaSuccess || !wptr)
+                return nfail(EMPSO_CUDA_ERROR, std::string("cudaGetSymbolAddress: ") + cudaGetErrorString(e));
+            g_ws_addr[dev] = wptr;
             g_scratch_addr[dev] = ptr;
         }
         base = static_cast<unsigned char *>(g_scratch_addr[dev]);
+        ws = g_ws_addr[dev];
     }
 
     // size check: the fixed part, the model fields and at least one slot
@@ -188,12 +200,11 @@ extern "C" empso_status eval_models_noalloc(const empso_grid *grid, const float 
                  "allocation-free path has %zu", probe.used + slot_bytes, M, NOALLOC_SCRATCH_BYTES);
         return nfail(EMPSO_UNSUPPORTED, buf);
     }
-    int sms = 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return nfail(EMPSO_CUDA_ERROR, "device attribute query failed");
-    const int per_sm = std::max(1, wave_max_ctas_per_sm(512));
     long long n_slots = (NOALLOC_SCRATCH_BYTES - probe.used) / slot_bytes;
-    n_slots = std::min<long long>({n_slots, n_inst, (long long)sms * per_sm});
+    n_slots = std::min<long long>({n_slots, n_inst, NOALLOC_FLIGHT});
+    const GridDev *gp = &g;
+    const WaveSplit split = wave_split(&gp, 1, g.R, n_inst, n_slots);
+    if (split.group < 1) return nfail(EMPSO_CUDA_ERROR, "occupancy of the streaming kernel");
     Layout L = carve(base, g, S, nrec_total, M, (int)n_slots);
     p.g.ex = L.ex;
     p.g.ez = L.ez;
@@ -208,9 +219,8 @@ extern "C" empso_status eval_models_noalloc(const empso_grid *grid, const float 
         (e = launch_grid_tables(p.g, L.ex, L.ez, L.wavelet, L.Wx, L.Wz, grid->vmax, grid->f0, st)) !=
             cudaSuccess ||
         (e = launch_vel_to_field(p.g, vel, M, L.fields, p.g.field, st)) != cudaSuccess ||
-        (e = cudaMemsetAsync(L.counter, 0, sizeof(int), st)) != cudaSuccess ||
-        (e = launch_wave(L.grid, L.insts, (int)n_inst, L.counter, L.slots, 2 * p.g.field, (int)n_slots,
-                         512, L.partial, st)) != cudaSuccess ||
+        (e = launch_wave(g.R, L.grid, L.insts, (int)n_inst, split, ws, L.slots, 2 * p.g.field, L.err, L.partial,
+                         st)) != cudaSuccess ||
         (e = launch_finalize(L.partial, L.weights, M, S, misfit, nullptr, st)) != cudaSuccess)
         return nfail(EMPSO_CUDA_ERROR, cudaGetErrorString(e));
     return EMPSO_OK;
