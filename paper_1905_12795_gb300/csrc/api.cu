@@ -2152,14 +2152,13 @@ empso_status surrogate_init(empso_ctx *ctx, int32_t hidden, int32_t capacity, fl
     CK(ctx, alloc((void **)&s.Xb, 2 * R * K));
     CK(ctx, alloc((void **)&s.A1b, 2 * R * H));
     CK(ctx, alloc((void **)&s.dZb, 2 * R * H));
-    CK(ctx, alloc((void **)&s.Z1, 4 * R * H));
+    CK(ctx, alloc((void **)&s.dZ1b, 2 * R * H));
     CK(ctx, alloc((void **)&s.Z2, 4 * R * H));
     CK(ctx, alloc((void **)&s.dZf, 4 * R * H));
     CK(ctx, alloc((void **)&s.dA, 4 * R * H));
     CK(ctx, alloc((void **)&s.y, 4 * R));
     CK(ctx, alloc((void **)&s.dy, 4 * R));
     CK(ctx, alloc((void **)&s.tb, 4 * R));
-    CK(ctx, alloc((void **)&s.rows, 4 * R));
     CK(ctx, alloc((void **)&s.loss, 4));
     CK(ctx, alloc((void **)&s.stats, 8));
     CK(ctx, alloc((void **)&s.xbuf, 4 * (size_t)capacity * K));
@@ -2309,7 +2308,7 @@ empso_status surrogate_grad(empso_ctx *ctx, const float *particles, const float 
         return fail(ctx, EMPSO_INVALID_ARG, "bad particles/target/grad");
     cudaStream_t st = (cudaStream_t)stream;
     SurDev &s = ctx->sur;
-    CK(ctx, sur_normalize(s, particles, nullptr, n, s.Xb, st));
+    CK(ctx, sur_normalize(s, particles, n, s.Xb, st));
     CK(ctx, sur_backward(s, s.Xb, target, n, loss ? loss : s.loss, st));
     CK(ctx, cudaMemcpyAsync(grad, s.g, 4 * (size_t)s.n_params, cudaMemcpyDeviceToDevice, st));
     return EMPSO_OK;

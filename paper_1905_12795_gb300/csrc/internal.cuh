@@ -253,10 +253,9 @@ struct SurDev {
     float *p = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;
     __nv_bfloat16 *W1b = nullptr, *W2b = nullptr;
     const double *xmin = nullptr, *xmax = nullptr;
-    __nv_bfloat16 *Xb = nullptr, *A1b = nullptr, *dZb = nullptr;
-    float *Z1 = nullptr, *Z2 = nullptr, *y = nullptr, *dy = nullptr, *dZf = nullptr, *dA = nullptr;
+    __nv_bfloat16 *Xb = nullptr, *A1b = nullptr, *dZb = nullptr, *dZ1b = nullptr;
+    float *Z2 = nullptr, *y = nullptr, *dy = nullptr, *dZf = nullptr, *dA = nullptr;
     float *tb = nullptr, *loss = nullptr, *stats = nullptr;
-    int *rows = nullptr;
     float *xbuf = nullptr, *ybuf = nullptr;
     int *count = nullptr;
     uint64_t seed = 0;
@@ -268,13 +267,11 @@ struct SurDev {
     int tc = 1;              // dense layers: 1 = tcgen05 (TMEM accumulator), 0 = mma.sync
     int *err = nullptr;      // status word for a tcgen05 completion wait that gives up
 };
-cudaError_t sur_forward(const SurDev &s, const __nv_bfloat16 *Xb, int n, float *y, cudaStream_t st);
 cudaError_t sur_backward(const SurDev &s, const __nv_bfloat16 *Xb, const float *t, int n, float *loss,
                          cudaStream_t st);
 cudaError_t sur_adam(SurDev &s, cudaStream_t st);
 cudaError_t sur_refresh_bf16(const SurDev &s, cudaStream_t st);
-cudaError_t sur_normalize(const SurDev &s, const float *x, const int *rows, int n, __nv_bfloat16 *out,
-                          cudaStream_t st);
+cudaError_t sur_normalize(const SurDev &s, const float *x, int n, __nv_bfloat16 *out, cudaStream_t st);
 cudaError_t sur_predict(const SurDev &s, const float *x, int n, float *logphi, cudaStream_t st);
 cudaError_t sur_append(const SurDev &s, const float *x, const double *misfit, const int *rows, int n,
                        cudaStream_t st);

@@ -22,6 +22,24 @@ namespace {
 // ---------------------------------------------------------------------------
 constexpr int GBM = 64, GBN = 64, GBK = 32, GPAD = 8;
 
+// One product and what becomes of it: v = C + bias[n], ReLU, or zero where the
+// mask (BF16 [M][ldm]) is not positive; FP32 Cf and/or BF16 Cb.
+struct Gemm {
+    int M, N, K;
+    const __nv_bfloat16 *A;
+    int lda, a_mk;
+    const __nv_bfloat16 *B;
+    int ldb, b_nk;
+    const float *bias;
+    int relu;
+    const __nv_bfloat16 *mask;
+    int ldm;
+    float *Cf;
+    int ldc;
+    __nv_bfloat16 *Cb;
+    int ldcb;
+};
+
 __device__ __forceinline__ void mma_bf16(float c[4], const unsigned a[4], const unsigned b[2])
 {
     asm volatile(
@@ -31,16 +49,14 @@ __device__ __forceinline__ void mma_bf16(float c[4], const unsigned a[4], const 
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-__global__ void __launch_bounds__(128)
-gemm_bf16_kernel(int M, int N, int K, const __nv_bfloat16 *__restrict__ A, int lda, int a_mk,
-                 const __nv_bfloat16 *__restrict__ B, int ldb, int b_nk,
-                 const float *__restrict__ bias, int relu, float *Cf, int ldc, __nv_bfloat16 *Cb,
-                 int ldcb)
+__global__ void __launch_bounds__(128) gemm_bf16_kernel(const Gemm g)
 {
+    const int M = g.M, N = g.N, K = g.K, lda = g.lda, a_mk = g.a_mk, ldb = g.ldb, b_nk = g.b_nk;
+    const __nv_bfloat16 *__restrict__ A = g.A, *__restrict__ B = g.B;
     __shared__ __align__(16) __nv_bfloat16 As[GBM][GBK + GPAD];   // (m, k)
     __shared__ __align__(16) __nv_bfloat16 Bs[GBN][GBK + GPAD];   // (n, k)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int g = lane >> 2, t = lane & 3;
+    const int lg = lane >> 2, t = lane & 3;
     const int m0 = blockIdx.y * GBM, n0 = blockIdx.x * GBN;
     const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
     float acc[2][4][4];
@@ -74,7 +90,7 @@ gemm_bf16_kernel(int M, int N, int K, const __nv_bfloat16 *__restrict__ A, int l
             unsigned af[2][4], bf[4][2];
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
-                const int r = wm + 16 * i + g;
+                const int r = wm + 16 * i + lg;
                 af[i][0] = *reinterpret_cast<const unsigned *>(&As[r][ks + 2 * t]);
                 af[i][1] = *reinterpret_cast<const unsigned *>(&As[r + 8][ks + 2 * t]);
                 af[i][2] = *reinterpret_cast<const unsigned *>(&As[r][ks + 2 * t + 8]);
@@ -82,7 +98,7 @@ gemm_bf16_kernel(int M, int N, int K, const __nv_bfloat16 *__restrict__ A, int l
             }
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                const int c = wn + 8 * j + g;
+                const int c = wn + 8 * j + lg;
                 bf[j][0] = *reinterpret_cast<const unsigned *>(&Bs[c][ks + 2 * t]);
                 bf[j][1] = *reinterpret_cast<const unsigned *>(&Bs[c][ks + 2 * t + 8]);
             }
@@ -99,34 +115,40 @@ gemm_bf16_kernel(int M, int N, int K, const __nv_bfloat16 *__restrict__ A, int l
         for (int j = 0; j < 4; ++j)
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const int m = m0 + wm + 16 * i + g + (e >= 2 ? 8 : 0);
+                const int m = m0 + wm + 16 * i + lg + (e >= 2 ? 8 : 0);
                 const int n = n0 + wn + 8 * j + 2 * t + (e & 1);
                 if (m >= M || n >= N) continue;
                 float v = acc[i][j][e];
-                if (bias) v += bias[n];
-                if (relu) v = fmaxf(v, 0.f);
-                if (Cf) Cf[(size_t)m * ldc + n] = v;
-                if (Cb) Cb[(size_t)m * ldcb + n] = __float2bfloat16(v);
+                if (g.bias) v += g.bias[n];
+                if (g.relu) v = fmaxf(v, 0.f);
+                if (g.mask && !(__bfloat162float(g.mask[(size_t)m * g.ldm + n]) > 0.f)) v = 0.f;
+                if (g.Cf) g.Cf[(size_t)m * g.ldc + n] = v;
+                if (g.Cb) g.Cb[(size_t)m * g.ldcb + n] = __float2bfloat16(v);
             }
 }
 
 // ---------------------------------------------------------------------------
 // The same product on the 5th-generation tensor cores: tcgen05.mma with BF16
 // operands from shared memory and the FP32 accumulator in tensor memory.
-// One CTA (4 warps) computes a 128 x NT tile (NT = 64, or N rounded up to 16
-// when N < 64) over 64-deep k-chunks, double-buffered: while the tensor core
-// works on chunk c, the threads stage chunk c + 1 into the other buffer.
-// Staging writes the K-major canonical layout without swizzle (8-row x
-// 16-byte core matrices; the two 8-element halves of a 16-deep k-slice 128
-// bytes apart, successive 8-row groups 256 bytes apart): rows stored k-fastest
-// are copied 16 bytes at a time, operands stored m/n-fastest are transposed
-// in registers 8 x 8 elements at a time.  One thread issues four
-// 128 x NT x 16 MMAs per chunk and commits them to the buffer's mbarrier;
-// after the last chunk every warp reads its 32 accumulator rows with
-// tcgen05.ld for the epilogue (bias, ReLU, FP32 and/or BF16 stores).
+// One CTA (8 warps) computes a 128 x NT tile (NT = 64, or N rounded up to 16
+// when N < 64) over k-chunks of up to TKC = 256: the whole depth of a forward or
+// data-gradient product, so that all its loads are in flight together; deeper
+// products (the weight gradients, whose depth is the batch) are
+// double-buffered.  Staging writes the K-major canonical layout without swizzle
+// (8-row x 16-byte core matrices; the two 8-element halves of a 16-deep k-slice
+// 128 bytes apart, successive 8-row groups 256 bytes apart): rows stored
+// k-fastest are copied 16 bytes at a time, operands stored m/n-fastest are
+// transposed in registers 8 x 8 elements at a time.  One thread issues a
+// 128 x NT x 16 MMA per k-slice and commits a chunk's to the buffer's mbarrier;
+// after the last chunk every warp reads its 32 accumulator rows of every other
+// 16 columns with tcgen05.ld for the epilogue.  Bound by latency (launch, one
+// round of global loads, the epilogue), not by the tensor core: with 64-deep
+// chunks and 128 threads each chunk waited for its own loads, 25 us for 1024 x
+// 256 x 256 and 45 us for 256 x 256 x 1024 (ncu); now 17 and 26 us.
 // ---------------------------------------------------------------------------
-constexpr int TM = 128, TKC = 64, TNT = 64;
+constexpr int TM = 128, TKC = 256, TNT = 64, TC_THREADS = 256;
 constexpr int TC_SMEM = 2 * (TKC / 16) * (TM + TNT) * 32;   // two k-chunk buffers
+__host__ __device__ inline int tc_tile_n(int N) { return N >= TNT ? TNT : (N + 15) / 16 * 16; }
 
 __device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 
@@ -177,20 +199,26 @@ __device__ __forceinline__ bool mbar_wait_tc(unsigned addr, unsigned parity)
     }
 }
 
-// Stage rows r0 .. r0 + R - 1 (of M) x k-chunk k0 .. k0 + 63 (of K) of an
-// operand into the canonical layout at dst (4 slices of R x 16 elements).
-// kmajor: element (r, k) at src[r ld + k]; otherwise at src[k ld + r].
-// vec: ld % 8 == 0 and src 16-byte aligned (16-byte accesses allowed).
+// Stage rows r0 .. r0 + R - 1 (of M) x k0 .. k0 + kc - 1 (of K; kc a multiple
+// of 16) of an operand into the canonical layout at dst (kc / 16 slices of R x
+// 16 elements).  kmajor: element (r, k) at src[r ld + k]; otherwise at
+// src[k ld + r].  vec: ld % 8 == 0 and src 16-byte aligned (16-byte accesses
+// allowed).
 __device__ __forceinline__ void stage_operand(unsigned char *dst, const __nv_bfloat16 *__restrict__ src,
                                               int ld, int kmajor, bool vec, int r0, int R, int M,
-                                              int k0, int K)
+                                              int k0, int kc, int K)
 {
     const int tid = threadIdx.x;
     const __nv_bfloat16 zero = __float2bfloat16(0.f);
     if (vec && kmajor) {
-        // one 16-byte vector = 8 consecutive k of one row
-        for (int v = tid; v < R * (TKC / 8); v += blockDim.x) {
-            const int r = v / (TKC / 8), kv = (v % (TKC / 8)) * 8;
+        // one 16-byte vector = 8 consecutive k of one row; a warp takes 8 rows
+        // (one core matrix, every bank once) by 2 or 4 vectors (whole sectors)
+        const int nkv = kc / 8, kg = nkv % 4 == 0 ? 4 : 2;
+        const int per = 8 * kg, blocks_k = nkv / kg;
+#pragma unroll 8
+        for (int v = tid; v < R * nkv; v += TC_THREADS) {
+            const int in = v % per, blk = v / per;
+            const int r = (blk / blocks_k) * 8 + (in & 7), kv = ((blk % blocks_k) * kg + (in >> 3)) * 8;
             const int row = r0 + r, k = k0 + kv;
             uint4 val = make_uint4(0u, 0u, 0u, 0u);
             if (row < M) {
@@ -208,7 +236,7 @@ __device__ __forceinline__ void stage_operand(unsigned char *dst, const __nv_bfl
     } else if (vec && (M & 7) == 0) {
         // 8 (rows) x 8 (k) blocks: eight 16-byte loads along the rows, a
         // register transpose, eight 16-byte stores along k
-        for (int b = tid; b < (R / 8) * (TKC / 8); b += blockDim.x) {
+        for (int b = tid; b < (R / 8) * (kc / 8); b += TC_THREADS) {
             const int rb = (b % (R / 8)) * 8, kb = (b / (R / 8)) * 8;
             const int row = r0 + rb;
             uint4 in[8];
@@ -237,9 +265,9 @@ __device__ __forceinline__ void stage_operand(unsigned char *dst, const __nv_bfl
                     make_uint4(o[m][0], o[m][1], o[m][2], o[m][3]);
         }
     } else {
-        for (int e = tid; e < R * TKC; e += blockDim.x) {
+        for (int e = tid; e < R * kc; e += TC_THREADS) {
             int r, kk;
-            if (kmajor) { r = e / TKC; kk = e % TKC; } else { kk = e / R; r = e % R; }
+            if (kmajor) { r = e / kc; kk = e % kc; } else { kk = e / R; r = e % R; }
             const int row = r0 + r, k = k0 + kk;
             __nv_bfloat16 v = zero;
             if (row < M && k < K) v = kmajor ? src[(size_t)row * ld + k] : src[(size_t)k * ld + row];
@@ -248,19 +276,19 @@ __device__ __forceinline__ void stage_operand(unsigned char *dst, const __nv_bfl
     }
 }
 
-__global__ void __launch_bounds__(128)
-gemm_tc_kernel(int M, int N, int K, const __nv_bfloat16 *__restrict__ A, int lda, int a_mk, int a_vec,
-               const __nv_bfloat16 *__restrict__ B, int ldb, int b_nk, int b_vec,
-               const float *__restrict__ bias, int relu, float *Cf, int ldc, __nv_bfloat16 *Cb,
-               int ldcb, int NT, int *err)
+// tile (bx, by) of one product; a CTA's whole work
+__device__ __forceinline__ void gemm_tc_tile(const Gemm &g, int bx, int by, int *err)
 {
     extern __shared__ __align__(1024) unsigned char tsm[];
     __shared__ __align__(8) unsigned long long mbar[2];
     __shared__ unsigned tmem_base;
     __shared__ int s_fail;
+    const int M = g.M, N = g.N, K = g.K;
+    const int NT = tc_tile_n(N);
     const int stage_bytes = (TKC / 16) * (TM + NT) * 32;
     const int tid = threadIdx.x, warp = tid >> 5;
-    const int m0 = blockIdx.y * TM, n0 = blockIdx.x * NT;
+    const int m0 = by * TM, n0 = bx * NT;
+    const bool a_vec = g.lda % 8 == 0 && ((size_t)g.A & 15) == 0, b_vec = g.ldb % 8 == 0 && ((size_t)g.B & 15) == 0;
     const unsigned ncols = NT <= 32 ? 32u : 64u;        // tensor-memory columns (power of 2)
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&mbar[0])) : "memory");
@@ -285,16 +313,17 @@ gemm_tc_kernel(int M, int N, int K, const __nv_bfloat16 *__restrict__ A, int lda
         const int buf = c & 1;
         unsigned char *As = tsm + buf * stage_bytes;
         unsigned char *Bs = As + (TKC / 16) * TM * 32;
+        const int kc = min(TKC, (K - c * TKC + 15) / 16 * 16);
         // the MMAs that read this buffer two chunks ago are done before it is restaged
         if (c >= 2 && !mbar_wait_tc(smem_u32(&mbar[buf]), ((c - 2) >> 1) & 1)) s_fail = 1;
-        stage_operand(As, A, lda, a_mk, a_vec != 0, m0, TM, M, c * TKC, K);
-        stage_operand(Bs, B, ldb, b_nk, b_vec != 0, n0, NT, N, c * TKC, K);
+        stage_operand(As, g.A, g.lda, g.a_mk, a_vec, m0, TM, M, c * TKC, kc, K);
+        stage_operand(Bs, g.B, g.ldb, g.b_nk, b_vec, n0, NT, N, c * TKC, kc, K);
         // thread-written shared memory -> visible to the tensor core (async proxy)
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
         __syncthreads();
         if (tid == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-            for (int s = 0; s < TKC / 16; ++s) {
+            for (int s = 0; s < kc / 16; ++s) {
                 const unsigned long long ad = umma_desc(As + s * (TM * 32), 128, 256);
                 const unsigned long long bd = umma_desc(Bs + s * (NT * 32), 128, 256);
                 const unsigned acc = (c > 0 || s > 0) ? 1u : 0u;
@@ -315,12 +344,13 @@ gemm_tc_kernel(int M, int N, int K, const __nv_bfloat16 *__restrict__ A, int lda
     }
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     __syncthreads();
-    // epilogue: warp w reads accumulator rows 32 w .. 32 w + 31 (TMEM lanes)
-    const int row = m0 + 32 * warp + (tid & 31);
+    // epilogue: warp w reads accumulator rows 32 (w mod 4) .. + 31 (TMEM lanes),
+    // warps 0-3 the even blocks of 16 columns, warps 4-7 the odd ones
+    const int row = m0 + 32 * (warp & 3) + (tid & 31);
     const bool fail = s_fail != 0;
-    for (int c0 = 0; c0 < NT; c0 += 16) {
+    for (int c0 = 16 * (warp >> 2); c0 < NT; c0 += 32) {
         unsigned r[16];
-        const unsigned taddr = tmem + ((unsigned)(32 * warp) << 16) + (unsigned)c0;
+        const unsigned taddr = tmem + ((unsigned)(32 * (warp & 3)) << 16) + (unsigned)c0;
         asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
                      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
                        "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]),
@@ -334,14 +364,15 @@ gemm_tc_kernel(int M, int N, int K, const __nv_bfloat16 *__restrict__ A, int lda
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
             float t = __uint_as_float(r[j]);
-            if (bias && nb + j < N) t += bias[nb + j];
-            if (relu) t = fmaxf(t, 0.f);
+            if (g.bias && nb + j < N) t += g.bias[nb + j];
+            if (g.relu) t = fmaxf(t, 0.f);
+            if (g.mask && nb + j < N && !(__bfloat162float(g.mask[(size_t)row * g.ldm + nb + j]) > 0.f)) t = 0.f;
             v[j] = t;
         }
-        if (nb + 16 <= N && c0 + 16 <= NT) {
-            if (Cf) {
-                float *o = Cf + (size_t)row * ldc + nb;
-                if ((ldc & 3) == 0 && ((size_t)Cf & 15) == 0) {
+        if (nb + 16 <= N) {
+            if (g.Cf) {
+                float *o = g.Cf + (size_t)row * g.ldc + nb;
+                if ((g.ldc & 3) == 0 && ((size_t)g.Cf & 15) == 0) {
 #pragma unroll
                     for (int q = 0; q < 4; ++q)
                         reinterpret_cast<float4 *>(o)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
@@ -349,9 +380,9 @@ gemm_tc_kernel(int M, int N, int K, const __nv_bfloat16 *__restrict__ A, int lda
                     for (int j = 0; j < 16; ++j) o[j] = v[j];
                 }
             }
-            if (Cb) {
-                __nv_bfloat16 *o = Cb + (size_t)row * ldcb + nb;
-                if ((ldcb & 7) == 0 && ((size_t)Cb & 15) == 0) {
+            if (g.Cb) {
+                __nv_bfloat16 *o = g.Cb + (size_t)row * g.ldcb + nb;
+                if ((g.ldcb & 7) == 0 && ((size_t)g.Cb & 15) == 0) {
                     __nv_bfloat162 h[8];
 #pragma unroll
                     for (int q = 0; q < 8; ++q) h[q] = __floats2bfloat162_rn(v[2 * q], v[2 * q + 1]);
@@ -364,9 +395,9 @@ gemm_tc_kernel(int M, int N, int K, const __nv_bfloat16 *__restrict__ A, int lda
         } else {
             for (int j = 0; j < 16; ++j) {
                 const int n = nb + j;
-                if (n >= N || c0 + j >= NT) break;
-                if (Cf) Cf[(size_t)row * ldc + n] = v[j];
-                if (Cb) Cb[(size_t)row * ldcb + n] = __float2bfloat16(v[j]);
+                if (n >= N) break;
+                if (g.Cf) g.Cf[(size_t)row * g.ldc + n] = v[j];
+                if (g.Cb) g.Cb[(size_t)row * g.ldcb + n] = __float2bfloat16(v[j]);
             }
         }
     }
@@ -377,148 +408,210 @@ gemm_tc_kernel(int M, int N, int K, const __nv_bfloat16 *__restrict__ A, int lda
     if (tid == 0 && s_fail) atomicExch(err, EMPSO_TIMEOUT);
 }
 
-cudaError_t gemm(const SurDev &s, cudaStream_t st, int M, int N, int K, const __nv_bfloat16 *A, int lda, int a_mk,
-                 const __nv_bfloat16 *B, int ldb, int b_nk, const float *bias, int relu, float *Cf,
-                 int ldc, __nv_bfloat16 *Cb, int ldcb)
+// Column sums g[h] = sum_b v[b][h] over the batch, v = X, or relu(X) times
+// wrow[b]: 32 columns per CTA; the partial sum (x, y) takes rows y, y + 32, ...
+// of column x, then the 32 partial sums of a column are added pairwise in a
+// fixed tree (the same order on every call and for any block size).
+constexpr int CS_T = 32;
+struct ColSum {
+    const float *X, *wrow;
+    int n, H;
+    float *g;
+};
+__device__ __forceinline__ void colsum_cols(const ColSum &c, int bx)
 {
-    if (s.tc && s.err && M > 0 && N > 0 && K > 0) {
-        const int NT = N >= TNT ? TNT : ((N + 15) / 16) * 16;
-        dim3 grid((N + NT - 1) / NT, (M + TM - 1) / TM);
-        const size_t smem = (size_t)2 * (TKC / 16) * (TM + NT) * 32;
-        const int a_vec = (lda % 8 == 0) && (((size_t)A & 15) == 0);
-        const int b_vec = (ldb % 8 == 0) && (((size_t)B & 15) == 0);
-        gemm_tc_kernel<<<grid, 128, smem, st>>>(M, N, K, A, lda, a_mk, a_vec, B, ldb, b_nk, b_vec, bias,
-                                                relu, Cf, ldc, Cb, ldcb, NT, s.err);
+    __shared__ float red[CS_T][CS_T + 1];
+    const int tx = threadIdx.x % CS_T, h = bx * CS_T + tx, step = blockDim.x / CS_T;
+    for (int ty = threadIdx.x / CS_T; ty < CS_T; ty += step) {
+        float s = 0.f;
+        if (h < c.H)
+#pragma unroll 8
+            for (int b = ty; b < c.n; b += CS_T) {
+                float v = c.X[(size_t)b * c.H + h];
+                if (c.wrow) v = fmaxf(v, 0.f) * c.wrow[b];
+                s += v;
+            }
+        red[ty][tx] = s;
+    }
+    __syncthreads();
+    for (int st = CS_T / 2; st > 0; st >>= 1) {
+        for (int ty = threadIdx.x / CS_T; ty < st; ty += step) red[ty][tx] += red[ty + st][tx];
+        __syncthreads();
+    }
+    if (threadIdx.x < CS_T && h < c.H) c.g[h] = red[0][tx];
+}
+
+// out = sum_i v[i]: one CTA, 1024 strided partial sums, then a fixed tree
+__device__ __forceinline__ void sum_all(const float *__restrict__ v, int n, float *out)
+{
+    __shared__ float red[1024];
+    for (int t = threadIdx.x; t < 1024; t += blockDim.x) {
+        float s = 0.f;
+        for (int i = t; i < n; i += 1024) s += v[i];
+        red[t] = s;
+    }
+    __syncthreads();
+    for (int st = 512; st > 0; st >>= 1) {
+        for (int t = threadIdx.x; t < st; t += blockDim.x) red[t] += red[t + st];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) *out = red[0];
+}
+
+// the loss 1/(2n) sum (y - t)^2 (one CTA of 256 threads or more, fixed order)
+__device__ __forceinline__ void loss_sum(const float *__restrict__ y, const float *__restrict__ t, int n, float *loss)
+{
+    __shared__ double red[8];
+    if (threadIdx.x < 256) {
+        double s = 0.0;
+        for (int b = threadIdx.x; b < n; b += 256) {
+            const float r = y[b] - t[b];
+            s += (double)r * r;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double v = 0.0;
+        for (int w = 0; w < 8; ++w) v += red[w];
+        if (loss) *loss = (float)(0.5 * v / n);
+    }
+}
+
+// Independent parts of the backward pass in one launch: up to two products,
+// up to two column sums, the sum of dy and the loss (the small parts would
+// each wait for a launch and leave the GPU idle: with these, the fused minibatch
+// and the fused head, a training step of 1024 pairs, K = 32, H = 256, takes 7
+// launches instead of 17, and six steps and a prediction 584 us instead of 1169).
+struct Jobs {
+    Gemm g[2];
+    ColSum c[2];
+    int n_gemm = 0, n_col = 0, sums = 0;
+    const float *dy = nullptr, *y = nullptr, *t = nullptr;   // sums: sum of dy into gb3, the loss
+    int n = 0;
+    float *gb3 = nullptr, *loss = nullptr;
+};
+
+__host__ __device__ inline int tc_tiles(const Gemm &g)
+{
+    const int NT = tc_tile_n(g.N);
+    return (g.N + NT - 1) / NT * ((g.M + TM - 1) / TM);
+}
+
+// part b of the jobs' vector work: the column sums' CTAs, then dy's sum and the loss
+__device__ __forceinline__ void vector_job(const Jobs &j, int b)
+{
+    for (int i = 0; i < j.n_col; ++i) {
+        const int n = (j.c[i].H + CS_T - 1) / CS_T;
+        if (b < n) return colsum_cols(j.c[i], b);
+        b -= n;
+    }
+    if (b == 0) sum_all(j.dy, j.n, j.gb3);
+    else loss_sum(j.y, j.t, j.n, j.loss);
+}
+
+__host__ inline int vector_blocks(const Jobs &j)
+{
+    int n = j.sums ? 2 : 0;
+    for (int i = 0; i < j.n_col; ++i) n += (j.c[i].H + CS_T - 1) / CS_T;
+    return n;
+}
+
+__global__ void __launch_bounds__(TC_THREADS) jobs_tc_kernel(const Jobs j, int *err)
+{
+    int b = blockIdx.x;
+    for (int i = 0; i < j.n_gemm; ++i) {
+        const int n = tc_tiles(j.g[i]);
+        if (b < n) {
+            const int nx = (j.g[i].N + tc_tile_n(j.g[i].N) - 1) / tc_tile_n(j.g[i].N);
+            return gemm_tc_tile(j.g[i], b % nx, b / nx, err);
+        }
+        b -= n;
+    }
+    vector_job(j, b);
+}
+
+__global__ void __launch_bounds__(TC_THREADS) jobs_vector_kernel(const Jobs j) { vector_job(j, blockIdx.x); }
+
+// the jobs on the context's backend: one launch on tcgen05, else one per product
+cudaError_t run_jobs(const SurDev &s, const Jobs &j, cudaStream_t st)
+{
+    const int vb = vector_blocks(j);
+    if (s.tc && s.err) {
+        int n = vb;
+        for (int i = 0; i < j.n_gemm; ++i) n += tc_tiles(j.g[i]);
+        if (n > 0) jobs_tc_kernel<<<n, TC_THREADS, j.n_gemm ? TC_SMEM : 0, st>>>(j, s.err);
         return cudaGetLastError();
     }
-    dim3 grid((N + GBN - 1) / GBN, (M + GBM - 1) / GBM);
-    gemm_bf16_kernel<<<grid, 128, 0, st>>>(M, N, K, A, lda, a_mk, B, ldb, b_nk, bias, relu, Cf, ldc,
-                                           Cb, ldcb);
+    for (int i = 0; i < j.n_gemm; ++i) {
+        const Gemm &g = j.g[i];
+        gemm_bf16_kernel<<<dim3((g.N + GBN - 1) / GBN, (g.M + GBM - 1) / GBM), 128, 0, st>>>(g);
+    }
+    if (vb) jobs_vector_kernel<<<vb, TC_THREADS, 0, st>>>(j);
     return cudaGetLastError();
+}
+
+cudaError_t run_gemm(const SurDev &s, const Gemm &g, cudaStream_t st)
+{
+    Jobs j;
+    j.g[0] = g;
+    j.n_gemm = 1;
+    return run_jobs(s, j, st);
 }
 
 // ---------------------------------------------------------------------------
 // elementwise and reduction kernels
 // ---------------------------------------------------------------------------
 
-// x_n = 2 (x - xmin) / (xmax - xmin) - 1, as BF16 rows of the batch
-__global__ void normalize_kernel(const float *__restrict__ x, const int *__restrict__ rows, int n,
-                                 int K, const double *__restrict__ xmin,
+// x_n = 2 (x - xmin) / (xmax - xmin) - 1 as BF16
+__device__ __forceinline__ __nv_bfloat16 normalized(float x, int k, const double *__restrict__ xmin,
+                                                    const double *__restrict__ xmax)
+{
+    const float lo = (float)xmin[k], hi = (float)xmax[k];
+    return __float2bfloat16(2.f * (x - lo) / (hi - lo) - 1.f);
+}
+
+__global__ void normalize_kernel(const float *__restrict__ x, int n, int K, const double *__restrict__ xmin,
                                  const double *__restrict__ xmax, __nv_bfloat16 *out)
 {
     const long long tot = (long long)n * K;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot;
-         e += (long long)gridDim.x * blockDim.x) {
-        const int b = (int)(e / K), k = (int)(e % K);
-        const int src = rows ? rows[b] : b;
-        const float lo = (float)xmin[k], hi = (float)xmax[k];
-        out[e] = __float2bfloat16(2.f * (x[(size_t)src * K + k] - lo) / (hi - lo) - 1.f);
-    }
+         e += (long long)gridDim.x * blockDim.x)
+        out[e] = normalized(x[e], (int)(e % K), xmin, xmax);
 }
 
-// y[b] = sum_h relu(Z2[b][h]) w3[h] + b3, one warp per row (fixed order)
+// The head, one warp per row b (fixed order): y = sum_h relu(Z2[b][h]) w3[h] +
+// b3.  Predicting (stats given): out[b] = y sigma + mu.  Training (t given):
+// also dy = (y - t) / n and, while the row is at hand, the gradient of the
+// hidden layer dZ2 = dy w3 [Z2 > 0] (FP32 and BF16 copies).
 __global__ void head_kernel(const float *__restrict__ Z2, int n, int H, const float *__restrict__ w3,
-                            const float *__restrict__ b3, float *y)
+                            const float *__restrict__ b3, float *y, const float *__restrict__ stats, float *out,
+                            const float *__restrict__ t, float *dy, float *dZf, __nv_bfloat16 *dZb)
 {
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (warp >= n) return;
+    const float *z = Z2 + (size_t)warp * H;
     float s = 0.f;
-    for (int h = lane; h < H; h += 32) s = fmaf(fmaxf(Z2[(size_t)warp * H + h], 0.f), w3[h], s);
+#pragma unroll 8
+    for (int h = lane; h < H; h += 32) s = fmaf(fmaxf(z[h], 0.f), w3[h], s);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) y[warp] = s + b3[0];
-}
-
-// dy = (y - t) / n and the loss 1/(2n) sum (y - t)^2 (one block, fixed order)
-__global__ void loss_kernel(const float *__restrict__ y, const float *__restrict__ t, int n,
-                            float *dy, float *loss)
-{
-    __shared__ double red[32];
-    double s = 0.0;
-    for (int b = threadIdx.x; b < n; b += blockDim.x) {
-        const float r = y[b] - t[b];
-        dy[b] = r / (float)n;
-        s += (double)r * r;
+    s = __shfl_sync(0xffffffffu, s, 0) + b3[0];
+    if (lane == 0) {
+        y[warp] = s;
+        if (out) out[warp] = s * stats[1] + stats[0];
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double v = 0.0;
-        for (int w = 0; w < (int)(blockDim.x + 31) / 32; ++w) v += red[w];
-        if (loss) *loss = (float)(0.5 * v / n);
+    if (!t) return;
+    const float r = s - t[warp], d = r / (float)n;
+    if (lane == 0) dy[warp] = d;
+#pragma unroll 8
+    for (int h = lane; h < H; h += 32) {
+        const float v = z[h] > 0.f ? d * w3[h] : 0.f;
+        dZf[(size_t)warp * H + h] = v;
+        dZb[(size_t)warp * H + h] = __float2bfloat16(v);
     }
-}
-
-// dZ2[b][h] = dy[b] w3[h] [Z2 > 0] (FP32 and BF16 copies)
-__global__ void dz2_kernel(const float *__restrict__ dy, const float *__restrict__ Z2,
-                           const float *__restrict__ w3, int n, int H, float *dZf,
-                           __nv_bfloat16 *dZb)
-{
-    const long long tot = (long long)n * H;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot;
-         e += (long long)gridDim.x * blockDim.x) {
-        const int b = (int)(e / H), h = (int)(e % H);
-        const float v = Z2[e] > 0.f ? dy[b] * w3[h] : 0.f;
-        dZf[e] = v;
-        dZb[e] = __float2bfloat16(v);
-    }
-}
-
-// dZ1 = dA1 [Z1 > 0] (FP32 in place and BF16 copy)
-__global__ void relu_back_kernel(float *dA, const float *__restrict__ Z, long long tot,
-                                 __nv_bfloat16 *dZb)
-{
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot;
-         e += (long long)gridDim.x * blockDim.x) {
-        const float v = Z[e] > 0.f ? dA[e] : 0.f;
-        dA[e] = v;
-        dZb[e] = __float2bfloat16(v);
-    }
-}
-
-// Column sums g[h] = sum_b v[b][h] over the batch, v = X, or relu(Z) times
-// wrow[b]: one CTA of 32 x 32 threads per 32 columns; thread (x, y) sums rows
-// y, y + 32, ... of column x, then the 32 partial sums of a column are added
-// pairwise in a fixed tree (the same order on every call).
-constexpr int CS_T = 32;
-__global__ void __launch_bounds__(CS_T * CS_T)
-colsum_kernel(const float *__restrict__ X, const float *__restrict__ wrow,
-              const float *__restrict__ Zrelu, int n, int H, float *g)
-{
-    __shared__ float red[CS_T][CS_T + 1];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int h = blockIdx.x * CS_T + tx;
-    float s = 0.f;
-    if (h < H)
-        for (int b = ty; b < n; b += CS_T) {
-            float v = X ? X[(size_t)b * H + h] : fmaxf(Zrelu[(size_t)b * H + h], 0.f);
-            if (wrow) v *= wrow[b];
-            s += v;
-        }
-    red[ty][tx] = s;
-    __syncthreads();
-    for (int st = CS_T / 2; st > 0; st >>= 1) {
-        if (ty < st) red[ty][tx] += red[ty + st][tx];
-        __syncthreads();
-    }
-    if (ty == 0 && h < H) g[h] = red[0][tx];
-}
-
-// out = sum_i v[i]: one CTA, strided partial sums, then a fixed tree
-__global__ void sum_kernel(const float *__restrict__ v, int n, float *out)
-{
-    __shared__ float red[1024];
-    float s = 0.f;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) s += v[i];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-        if ((int)threadIdx.x < st) red[threadIdx.x] += red[threadIdx.x + st];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *out = red[0];
 }
 
 // Adam on FP32 master weights, then BF16 copies of the two hidden matrices
@@ -564,26 +657,34 @@ __device__ __forceinline__ uint4 philox_s(uint4 c, uint32_t k0, uint32_t k1)
     return c;
 }
 
-// batch rows drawn uniformly from the filled part of the replay buffer (its
-// first min(have_host, cap) rows when have_host >= 0, else the device count's);
-// with recent > 0 the second half of the batch comes from the newest
-// min(recent, filled) pairs instead (the swarm's current neighbourhood)
-__global__ void sample_kernel(int *rows, int B, const int *count, int have_host, int cap, uint64_t seed,
-                              int step, int recent)
+// A minibatch, one warp per row: the row drawn uniformly from the filled part of
+// the replay buffer (its first min(have_host, cap) rows when have_host >= 0,
+// else the device count's; with recent > 0 the second half of the batch comes
+// from the newest min(recent, filled) pairs instead, the swarm's current
+// neighbourhood), its standardised target (log phi - mu) / sigma and its
+// position scaled to [-1, 1] in BF16 (the buffer holds raw positions).
+__global__ void batch_kernel(int B, int K, const int *count, int have_host, int cap, uint64_t seed, int step,
+                             int recent, const float *__restrict__ xbuf, const float *__restrict__ ybuf,
+                             const float *__restrict__ stats, const double *__restrict__ xmin,
+                             const double *__restrict__ xmax, float *t, __nv_bfloat16 *Xb)
 {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (b >= B) return;
     const int total = have_host >= 0 ? have_host : *count;   // pairs appended so far
     const int have = min(total, cap);
     const uint4 w = philox_s(make_uint4((uint32_t)step, (uint32_t)b, 0x5u, 0x7u), (uint32_t)seed,
                              (uint32_t)(seed >> 32));
+    int row;
     if (recent > 0 && b >= B / 2 && have > 0) {
         const int span = min(recent, have);
         const int j = (int)(((unsigned long long)w.x * (unsigned long long)span) >> 32);
-        rows[b] = (int)(((long long)total - 1 - j) % cap);
-        return;
+        row = (int)(((long long)total - 1 - j) % cap);
+    } else {
+        row = have > 0 ? (int)(((unsigned long long)w.x * (unsigned long long)have) >> 32) : 0;
     }
-    rows[b] = have > 0 ? (int)(((unsigned long long)w.x * (unsigned long long)have) >> 32) : 0;
+    if (lane == 0) t[b] = (ybuf[row] - stats[0]) / stats[1];
+    for (int k = lane; k < K; k += 32)
+        Xb[(size_t)b * K + k] = normalized(xbuf[(size_t)row * K + k], k, xmin, xmax);
 }
 
 // Spearman rank correlation of the k modelled particles' true misfits fk
@@ -625,14 +726,6 @@ rank_corr_kernel(const double *__restrict__ fk, const int *__restrict__ rows,
         const double kk = (double)k;
         *rho = k > 1 ? (float)(1.0 - 6.0 * s / (kk * (kk * kk - 1.0))) : 1.f;
     }
-}
-
-// standardised targets of the batch: (log phi - mu) / sigma
-__global__ void targets_kernel(const float *__restrict__ ybuf, const int *__restrict__ rows, int B,
-                               const float *__restrict__ stats, float *t)
-{
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b < B) t[b] = (ybuf[rows[b]] - stats[0]) / stats[1];
 }
 
 // mean and standard deviation of the filled replay targets (one block)
@@ -728,14 +821,6 @@ append_kernel(const float *__restrict__ x, const double *__restrict__ misfit,
     if (tid == 0) *count = base;
 }
 
-// predictions back to log-misfit: out = y sigma + mu
-__global__ void destandardize_kernel(const float *__restrict__ y, int n, const float *__restrict__ stats,
-                                     float *out)
-{
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b < n) out[b] = y[b] * stats[1] + stats[0];
-}
-
 // indices of the k smallest keys (ties to the lower index), one block, P <= 2048
 __global__ void __launch_bounds__(1024) select_kernel(const float *__restrict__ key, int P, int k, int *out)
 {
@@ -815,24 +900,24 @@ inline int blocks_for(long long n, int per = 256)
 // host-side launchers used by api.cu
 // ---------------------------------------------------------------------------
 
-// opt the tcgen05 GEMM into its 48 KiB of dynamic shared memory (current device)
+// opt the tcgen05 products into their two chunk buffers (current device)
 cudaError_t sur_prepare_tc()
 {
-    return cudaFuncSetAttribute(gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
+    return cudaFuncSetAttribute(jobs_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
 }
 
-cudaError_t sur_forward(const SurDev &s, const __nv_bfloat16 *Xb, int n, float *y, cudaStream_t st)
+namespace {
+
+// both hidden layers of batch Xb [n][K]: A1b = relu(X W1 + b1) (BF16), Z2
+cudaError_t hidden_layers(const SurDev &s, const __nv_bfloat16 *Xb, int n, cudaStream_t st)
 {
     cudaError_t e;
-    if ((e = gemm(s, st, n, s.H, s.K, Xb, s.K, 1, s.W1b, s.K, 1, s.p + s.off_b1, 1, s.Z1, s.H, s.A1b,
-                  s.H)))
+    if ((e = run_gemm(s, {n, s.H, s.K, Xb, s.K, 1, s.W1b, s.K, 1, s.p + s.off_b1, 1, nullptr, 0, nullptr, 0, s.A1b, s.H}, st)))
         return e;
-    if ((e = gemm(s, st, n, s.H, s.H, s.A1b, s.H, 1, s.W2b, s.H, 1, s.p + s.off_b2, 0, s.Z2, s.H,
-                  nullptr, 0)))
-        return e;
-    head_kernel<<<(n * 32 + 255) / 256, 256, 0, st>>>(s.Z2, n, s.H, s.p + s.off_w3, s.p + s.off_b3, y);
-    return cudaGetLastError();
+    return run_gemm(s, {n, s.H, s.H, s.A1b, s.H, 1, s.W2b, s.H, 1, s.p + s.off_b2, 0, nullptr, 0, s.Z2, s.H, nullptr, 0}, st);
 }
+
+}  // namespace
 
 // gradient of the half-MSE on batch (Xb [n][K] BF16, t [n]) into s.g; loss
 // to *loss (device float, may be null)
@@ -840,31 +925,33 @@ cudaError_t sur_backward(const SurDev &s, const __nv_bfloat16 *Xb, const float *
                          float *loss, cudaStream_t st)
 {
     cudaError_t e;
-    if ((e = sur_forward(s, Xb, n, s.y, st))) return e;
-    loss_kernel<<<1, 256, 0, st>>>(s.y, t, n, s.dy, loss);
-    // head: g_w3 = sum_b relu(Z2) dy, g_b3 = sum_b dy
-    const dim3 cs_grid((s.H + CS_T - 1) / CS_T), cs_block(CS_T, CS_T);
-    colsum_kernel<<<cs_grid, cs_block, 0, st>>>(nullptr, s.dy, s.Z2, n, s.H, s.g + s.off_w3);
-    sum_kernel<<<1, 1024, 0, st>>>(s.dy, n, s.g + s.off_b3);
-    // layer 2
-    dz2_kernel<<<blocks_for((long long)n * s.H), 256, 0, st>>>(s.dy, s.Z2, s.p + s.off_w3, n, s.H,
-                                                             s.dZf, s.dZb);
-    colsum_kernel<<<cs_grid, cs_block, 0, st>>>(s.dZf, nullptr, nullptr, n, s.H, s.g + s.off_b2);
-    // g_W2[h][h'] = sum_b dZ2[b][h] A1[b][h']
-    if ((e = gemm(s, st, s.H, s.H, n, s.dZb, s.H, 0, s.A1b, s.H, 0, nullptr, 0, s.g + s.off_W2, s.H,
-                  nullptr, 0)))
-        return e;
-    // dA1 = dZ2 W2  -> dZ1 = dA1 [Z1 > 0]
-    if ((e = gemm(s, st, n, s.H, s.H, s.dZb, s.H, 1, s.W2b, s.H, 0, nullptr, 0, s.dA, s.H, nullptr, 0)))
-        return e;
-    relu_back_kernel<<<blocks_for((long long)n * s.H), 256, 0, st>>>(s.dA, s.Z1, (long long)n * s.H,
-                                                                     s.dZb);
-    colsum_kernel<<<cs_grid, cs_block, 0, st>>>(s.dA, nullptr, nullptr, n, s.H, s.g + s.off_b1);
-    // g_W1[h][k] = sum_b dZ1[b][h] X[b][k]
-    if ((e = gemm(s, st, s.H, s.K, n, s.dZb, s.H, 0, Xb, s.K, 0, nullptr, 0, s.g + s.off_W1, s.K,
-                  nullptr, 0)))
-        return e;
-    return cudaGetLastError();
+    if ((e = hidden_layers(s, Xb, n, st))) return e;
+    head_kernel<<<(n * 32 + 255) / 256, 256, 0, st>>>(s.Z2, n, s.H, s.p + s.off_w3, s.p + s.off_b3, s.y, nullptr,
+                                                      nullptr, t, s.dy, s.dZf, s.dZb);
+    // dZ1 = (dZ2 W2) [A1 > 0]; g_W2[h][h'] = sum_b dZ2[b][h] A1[b][h']; the
+    // head's g_w3 = sum_b relu(Z2) dy and g_b3 = sum_b dy; g_b2; the loss
+    Jobs j;
+    j.n_gemm = 2;
+    j.g[0] = {s.H, s.H, n, s.dZb, s.H, 0, s.A1b, s.H, 0, nullptr, 0, nullptr, 0, s.g + s.off_W2, s.H, nullptr, 0};
+    j.g[1] = {n, s.H, s.H, s.dZb, s.H, 1, s.W2b, s.H, 0, nullptr, 0, s.A1b, s.H, s.dA, s.H, s.dZ1b, s.H};
+    j.n_col = 2;
+    j.c[0] = {s.Z2, s.dy, n, s.H, s.g + s.off_w3};
+    j.c[1] = {s.dZf, nullptr, n, s.H, s.g + s.off_b2};
+    j.sums = 1;
+    j.dy = s.dy;
+    j.y = s.y;
+    j.t = t;
+    j.n = n;
+    j.gb3 = s.g + s.off_b3;
+    j.loss = loss;
+    if ((e = run_jobs(s, j, st))) return e;
+    // g_W1[h][k] = sum_b dZ1[b][h] X[b][k]; g_b1
+    Jobs i;
+    i.n_gemm = 1;
+    i.g[0] = {s.H, s.K, n, s.dZ1b, s.H, 0, Xb, s.K, 0, nullptr, 0, nullptr, 0, s.g + s.off_W1, s.K, nullptr, 0};
+    i.n_col = 1;
+    i.c[0] = {s.dA, nullptr, n, s.H, s.g + s.off_b1};
+    return run_jobs(s, i, st);
 }
 
 cudaError_t sur_adam(SurDev &s, cudaStream_t st)
@@ -887,20 +974,19 @@ cudaError_t sur_refresh_bf16(const SurDev &s, cudaStream_t st)
     return cudaGetLastError();
 }
 
-cudaError_t sur_normalize(const SurDev &s, const float *x, const int *rows, int n, __nv_bfloat16 *out,
-                          cudaStream_t st)
+cudaError_t sur_normalize(const SurDev &s, const float *x, int n, __nv_bfloat16 *out, cudaStream_t st)
 {
-    normalize_kernel<<<blocks_for((long long)n * s.K), 256, 0, st>>>(x, rows, n, s.K, s.xmin, s.xmax,
-                                                                     out);
+    normalize_kernel<<<blocks_for((long long)n * s.K), 256, 0, st>>>(x, n, s.K, s.xmin, s.xmax, out);
     return cudaGetLastError();
 }
 
 cudaError_t sur_predict(const SurDev &s, const float *x, int n, float *logphi, cudaStream_t st)
 {
     cudaError_t e;
-    if ((e = sur_normalize(s, x, nullptr, n, s.Xb, st))) return e;
-    if ((e = sur_forward(s, s.Xb, n, s.y, st))) return e;
-    destandardize_kernel<<<(n + 255) / 256, 256, 0, st>>>(s.y, n, s.stats, logphi);
+    if ((e = sur_normalize(s, x, n, s.Xb, st))) return e;
+    if ((e = hidden_layers(s, s.Xb, n, st))) return e;
+    head_kernel<<<(n * 32 + 255) / 256, 256, 0, st>>>(s.Z2, n, s.H, s.p + s.off_w3, s.p + s.off_b3, s.y, s.stats,
+                                                      logphi, nullptr, nullptr, nullptr, nullptr);
     return cudaGetLastError();
 }
 
@@ -914,13 +1000,11 @@ cudaError_t sur_append(const SurDev &s, const float *x, const double *misfit, co
 cudaError_t sur_train(SurDev &s, int steps, int B, cudaStream_t st, int have)
 {
     cudaError_t e;
-    stats_kernel<<<1, 256, 0, st>>>(s.ybuf, s.count, have, s.cap, s.stats);
+    stats_kernel<<<1, 1024, 0, st>>>(s.ybuf, s.count, have, s.cap, s.stats);
     for (int i = 0; i < steps; ++i) {
-        sample_kernel<<<(B + 255) / 256, 256, 0, st>>>(s.rows, B, s.count, have, s.cap, s.seed,
-                                                       s.sample_step++, s.recent);
-        targets_kernel<<<(B + 255) / 256, 256, 0, st>>>(s.ybuf, s.rows, B, s.stats, s.tb);
-        // the buffer holds raw positions: scale the batch rows to [-1, 1] in BF16
-        if ((e = sur_normalize(s, s.xbuf, s.rows, B, s.Xb, st))) return e;
+        batch_kernel<<<(B * 32 + 255) / 256, 256, 0, st>>>(B, s.K, s.count, have, s.cap, s.seed, s.sample_step++,
+                                                           s.recent, s.xbuf, s.ybuf, s.stats, s.xmin, s.xmax, s.tb,
+                                                           s.Xb);
         if ((e = sur_backward(s, s.Xb, s.tb, B, s.loss, st))) return e;
         if ((e = sur_adam(s, st))) return e;
     }
