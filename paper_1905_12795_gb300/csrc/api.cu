@@ -1057,8 +1057,8 @@ empso_status empso_create(const empso_grid *grids, int32_t ngrids, const float *
         ctx->has_pso = true;
         ctx->pcfg = p;
         const size_t PD = (size_t)p.P * p.D;
-        if ((rc = ck(cudaMalloc(&ctx->pso_mem, sizeof(double) * (3 * PD + p.P + 2 * p.D)), "swarm")) ||
-            (rc = ck(cudaMalloc(&ctx->pso_int, sizeof(int) * (2 * p.P + 2)), "swarm ints")) ||
+        if ((rc = ck(cudaMalloc(&ctx->pso_mem, sizeof(double) * (3 * PD + p.P + 2 * p.D + 1)), "swarm")) ||
+            (rc = ck(cudaMalloc(&ctx->pso_int, sizeof(int) * (2 * p.P + 3)), "swarm ints")) ||
             (rc = ck(cudaMalloc(&ctx->xf, sizeof(float) * PD), "positions")) ||
             (rc = ck(cudaMalloc(&ctx->gen_misfit, sizeof(double) * p.P), "generation misfit")))
             return bail(rc);
@@ -1080,14 +1080,16 @@ empso_status empso_create(const empso_grid *grids, int32_t ngrids, const float *
         double *bounds = s.pf + p.P;
         s.xmin = bounds;
         s.xmax = bounds + p.D;
+        s.chi = bounds + 2 * p.D;
         s.order = ctx->pso_int;
         s.gk = ctx->pso_int + p.P;
         s.rank_of = ctx->pso_int + p.P + 2;
+        s.k_new = ctx->pso_int + 2 * p.P + 2;
         s.xf = ctx->xf;
         if ((rc = ck(cudaMemcpy(bounds, xmin, sizeof(double) * p.D, cudaMemcpyHostToDevice), "xmin")) ||
             (rc = ck(cudaMemcpy(bounds + p.D, xmax, sizeof(double) * p.D, cudaMemcpyHostToDevice),
                      "xmax")) ||
-            (rc = ck(cudaMemset(ctx->pso_int, 0, sizeof(int) * (2 * p.P + 2)), "swarm ints")))
+            (rc = ck(cudaMemset(ctx->pso_int, 0, sizeof(int) * (2 * p.P + 3)), "swarm ints")))
             return bail(rc);
     }
     if ((rc = ck(cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking), "capture stream")) ||
@@ -1719,17 +1721,7 @@ empso_status pso_get_state(empso_ctx *ctx, double *x, double *v, double *p, doub
     ctx->err.clear();
     if (!ctx->has_pso) return fail(ctx, EMPSO_NOT_INITIALIZED, "context has no swarm");
     cudaStream_t st = (cudaStream_t)stream;
-    const size_t PD = sizeof(double) * ctx->pso.P * ctx->pso.D;
-    if (x) CK(ctx, cudaMemcpyAsync(x, ctx->pso.x, PD, cudaMemcpyDeviceToDevice, st));
-    if (v) CK(ctx, cudaMemcpyAsync(v, ctx->pso.v, PD, cudaMemcpyDeviceToDevice, st));
-    if (p) CK(ctx, cudaMemcpyAsync(p, ctx->pso.p, PD, cudaMemcpyDeviceToDevice, st));
-    if (pf)
-        CK(ctx, cudaMemcpyAsync(pf, ctx->pso.pf, sizeof(double) * ctx->pso.P,
-                                cudaMemcpyDeviceToDevice, st));
-    if (order)
-        CK(ctx, cudaMemcpyAsync(order, ctx->pso.order, sizeof(int) * ctx->pso.P,
-                                cudaMemcpyDeviceToDevice, st));
-    if (gk) CK(ctx, cudaMemcpyAsync(gk, ctx->pso.gk, 2 * sizeof(int), cudaMemcpyDeviceToDevice, st));
+    CK(ctx, launch_pso_state(ctx->pso, x, v, p, pf, order, gk, st));
     return EMPSO_OK;
 }
 

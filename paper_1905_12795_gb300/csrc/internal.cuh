@@ -237,12 +237,16 @@ struct PsoDev {
     double *pf;                  // [P]
     int *order;                  // [P]
     int *gk;                     // {g, k}
+    int *k_new;                  // generation of the step in progress
+    double *chi;                 // constriction factor, likewise
     int *rank_of;                // [P] EM rank of each particle in the current step
     float *xf;                   // [P][D] float copy of x (what generations evaluate)
 };
 cudaError_t launch_pso_init(const PsoDev &s, float *particles_out, cudaStream_t st);
 cudaError_t launch_pso_step(const PsoDev &s, const double *misfit, float *particles_out,
                             cudaStream_t st, const double *rank = nullptr);
+cudaError_t launch_pso_state(const PsoDev &s, double *x, double *v, double *p, double *pf, int *order, int *gk,
+                             cudaStream_t st);
 cudaError_t launch_xf_from_x(const PsoDev &s, cudaStream_t st);
 
 // Surrogate network (surrogate.cu): flat FP32 parameters in the order

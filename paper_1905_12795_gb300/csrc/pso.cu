@@ -169,65 +169,106 @@ __global__ void pso_init_kernel(PsoDev s, float *particles_out)
     }
 }
 
-constexpr int STEP_THREADS = 1024;
+constexpr int STEP_THREADS = 256, STEP_WARPS = STEP_THREADS / 32;
 
-// (key, index) lexicographic order: ties go to the lower index, which makes
-// the bitonic sort equivalent to a stable sort of the keys.
-__device__ __forceinline__ bool before(double fa, int ia, double fb, int ib)
+// (key, index) lexicographic order: ties go to the lower index
+__device__ __forceinline__ bool before(long long fa, int ia, long long fb, int ib)
 {
     return fa < fb || (fa == fb && ia < ib);
 }
 
-// One generation, first part, in one CTA: personal bests, global best and the
-// EM sort; the rank of every particle goes to s.rank_of for the second part.
-__global__ void __launch_bounds__(STEP_THREADS)
-pso_rank_kernel(PsoDev s, const double *misfit, const double *rank)
+// A key as an integer of the same order (-0 as +0; not a number after +inf):
+// integer comparisons run at the full rate, FP64 ones at 1/64 of it
+constexpr long long NO_NUMBER = 0x7fffffffffffffffLL;
+__device__ __forceinline__ long long ordered(double f)
 {
-    __shared__ double key[MAX_PSO_P];
-    __shared__ int idx[MAX_PSO_P];
-    __shared__ double bf[STEP_THREADS / 32];
-    __shared__ int bi[STEP_THREADS / 32];
-    const int tid = threadIdx.x;
-    const int P = s.P, D = s.D;
+    const long long b = __double_as_longlong(f), m = b & 0x7fffffffffffffffLL;
+    if (m > 0x7ff0000000000000LL) return NO_NUMBER;
+    return b < 0 ? -m : m;
+}
+
+// One generation, first part, one warp per particle over the whole GPU: the
+// personal best, and the particle's rank in the EM sort by counting the keys
+// before its own, (key, index) in lexicographic order: the position a stable
+// ascending sort gives it.  Every CTA keeps all keys in shared memory.  (One
+// CTA that updated every best and sorted bitonically, 55 passes over shared
+// memory for 1024 keys, took 53 us under ncu for P = 1024, D = 32; this takes
+// @RANKT@.)  The generation counter is not written here, where every CTA reads
+// it: the new one goes to s.k_new for the second part, beside the constriction
+// factor (Eq. 3), whose FP64 root and quotient every thread of the second part
+// would otherwise repeat.
+__global__ void __launch_bounds__(STEP_THREADS) pso_rank_kernel(PsoDev s, const double *misfit, const double *rank)
+{
+    __shared__ long long key[MAX_PSO_P];
+    const int P = s.P, D = s.D, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const double inf = __longlong_as_double(0x7ff0000000000000LL);
     const int k = s.gk[1] + 1;
-
-    // 1-2. fitness (non-finite -> +inf) and strict personal-best update
-    int N = 1;
-    while (N < P) N <<= 1;
-    for (int i = tid; i < N; i += STEP_THREADS) {
-        if (i < P) {
-            double f = misfit[i];
-            if (!isfinite(f)) f = inf;
-            // EM sort key: the fitness, or the given rank key (surrogate pre-screen)
-            double r = rank ? rank[i] : misfit[i];
-            if (!isfinite(r)) r = inf;
-            key[i] = r;
-            idx[i] = i;
-            if (f < s.pf[i]) {
-                s.pf[i] = f;
-                for (int d = 0; d < D; ++d) s.p[(size_t)i * D + d] = s.x[(size_t)i * D + d];
-            }
-        } else {
-            key[i] = inf;
-            idx[i] = 0x7fffffff;
+    const bool em = s.em_enabled && k >= s.em_start && s.NM > 0;
+    if (em) {
+        // EM sort key: the fitness, or the given rank key (surrogate pre-screen)
+        for (int i = threadIdx.x; i < P; i += STEP_THREADS) {
+            const double r = rank ? rank[i] : misfit[i];
+            key[i] = ordered(isfinite(r) ? r : inf);
         }
+        __syncthreads();
     }
-    __syncthreads();
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {   // a CTA without particles
+        *s.k_new = k;
+        const double phi = s.c1 + s.c2;
+        *s.chi = 2.0 / fabs(2.0 - phi - sqrt(phi * phi - 4.0 * phi));
+    }
+    const int i = blockIdx.x * STEP_WARPS + warp;
+    if (i >= P) return;
+    // fitness (non-finite -> +inf) and strict personal-best update
+    double f = misfit[i];
+    if (!isfinite(f)) f = inf;
+    const bool better = f < s.pf[i];
+    __syncwarp();
+    if (better) {
+        if (lane == 0) s.pf[i] = f;
+        for (int d = lane; d < D; d += 32) s.p[(size_t)i * D + d] = s.x[(size_t)i * D + d];
+    }
+    if (em) {
+        const long long own = key[i];
+        int r = 0;
+        for (int j = lane; j < P; j += 32) {
+            const long long o = key[j];
+            r += o < own || (o == own && j < i);
+        }
+        r = __reduce_add_sync(0xffffffffu, r);
+        if (lane == 0) {
+            s.rank_of[i] = r;
+            s.order[r] = i;
+        }
+    } else if (lane == 0) {
+        s.rank_of[i] = 0;
+        s.order[i] = i;
+    }
+}
 
-    // 3. global best: lowest-index argmin of pf
-    double bv = inf;
+// One generation, second part, one thread per (particle, node) over the whole
+// GPU: the global best (the lowest-index argmin of pf, found by every CTA for
+// itself: 8 KB of L2 reads for P = 1024 instead of another launch), then EM on
+// the NM worst, Eq. 1 / Eq. 2 with clamps on the rest.  Every element's
+// arithmetic is independent of the others', so spreading them over CTAs
+// changes no bit of the result.
+__global__ void __launch_bounds__(STEP_THREADS) pso_move_kernel(PsoDev s, float *particles_out)
+{
+    __shared__ long long bf[STEP_WARPS];
+    __shared__ int bi[STEP_WARPS];
+    const int P = s.P, D = s.D, tid = threadIdx.x;
+    long long bv = NO_NUMBER;
     int bj = 0x7fffffff;
     for (int i = tid; i < P; i += STEP_THREADS) {
-        const double v = s.pf[i];
-        if (before(v, i, bv, bj)) {
+        const long long v = ordered(s.pf[i]);
+        if (v != NO_NUMBER && before(v, i, bv, bj)) {
             bv = v;
             bj = i;
         }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        const double ov = __shfl_down_sync(0xffffffffu, bv, o);
+        const long long ov = __shfl_down_sync(0xffffffffu, bv, o);
         const int oj = __shfl_down_sync(0xffffffffu, bj, o);
         if (before(ov, oj, bv, bj)) {
             bv = ov;
@@ -239,71 +280,26 @@ pso_rank_kernel(PsoDev s, const double *misfit, const double *rank)
         bi[tid >> 5] = bj;
     }
     __syncthreads();
-    if (tid == 0) {
-        double v = bf[0];
-        int j = bi[0];
-        for (int w = 1; w < STEP_THREADS / 32; ++w)
-            if (before(bf[w], bi[w], v, j)) {
-                v = bf[w];
-                j = bi[w];
-            }
-        // all-infinite pf: every index ties, the lowest one wins (every
-        // thread read gk before the barrier above)
-        s.gk[0] = (j == 0x7fffffff) ? 0 : j;
+    bv = bf[0];
+    bj = bi[0];
+    for (int w = 1; w < STEP_WARPS; ++w)
+        if (before(bf[w], bi[w], bv, bj)) {
+            bv = bf[w];
+            bj = bi[w];
+        }
+    // no number among the fitnesses: the lowest index
+    const int g = bj == 0x7fffffff ? 0 : bj, k = *s.k_new;
+    if (blockIdx.x == 0 && tid == 0) {
+        s.gk[0] = g;
         s.gk[1] = k;
     }
-
-    // 4. EM: stable ascending sort of the fitness (bitonic on (f, i) pairs)
-    const bool em = s.em_enabled && k >= s.em_start && s.NM > 0;
-    if (em) {
-        for (int size = 2; size <= N; size <<= 1) {
-            for (int stride = size >> 1; stride > 0; stride >>= 1) {
-                for (int t = tid; t < N / 2; t += STEP_THREADS) {
-                    const int lo = 2 * t - (t & (stride - 1));
-                    const int hi = lo + stride;
-                    const bool up = (lo & size) == 0;
-                    const bool swap = up ? before(key[hi], idx[hi], key[lo], idx[lo])
-                                         : before(key[lo], idx[lo], key[hi], idx[hi]);
-                    if (swap) {
-                        const double tk = key[lo];
-                        key[lo] = key[hi];
-                        key[hi] = tk;
-                        const int ti = idx[lo];
-                        idx[lo] = idx[hi];
-                        idx[hi] = ti;
-                    }
-                }
-                __syncthreads();
-            }
-        }
-        for (int r = tid; r < P; r += STEP_THREADS) {
-            s.rank_of[idx[r]] = r;
-            s.order[r] = idx[r];
-        }
-    } else {
-        for (int r = tid; r < P; r += STEP_THREADS) {
-            s.rank_of[r] = 0;
-            s.order[r] = r;
-        }
-    }
-}
-
-// One generation, second part, one thread per (particle, node) over the whole
-// GPU: EM on the NM worst, Eq. 1 / Eq. 2 with clamps on the rest.  Every
-// element's arithmetic is independent of the others', so spreading them over
-// CTAs changes no bit of the result.
-__global__ void pso_move_kernel(PsoDev s, float *particles_out)
-{
-    const int P = s.P, D = s.D;
-    const int g = s.gk[0], k = s.gk[1];
     const int NM = s.NM;
     const bool em = s.em_enabled && k >= s.em_start && NM > 0;
-    const double phi = s.c1 + s.c2;
-    const double chi = 2.0 / fabs(2.0 - phi - sqrt(phi * phi - 4.0 * phi));
+    const double chi = *s.chi;
     const double *gx = s.p + (size_t)g * D;
     const long long total = (long long)P * D;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-         e += (long long)gridDim.x * blockDim.x) {
+    for (long long e = blockIdx.x * (long long)STEP_THREADS + tid; e < total;
+         e += (long long)gridDim.x * STEP_THREADS) {
         const int i = (int)(e / D), d = (int)(e % D);
         const double lo = s.xmin[d], hi = s.xmax[d];
         const double vr = hi - lo;
@@ -361,13 +357,44 @@ cudaError_t launch_xf_from_x(const PsoDev &s, cudaStream_t st)
 cudaError_t launch_pso_step(const PsoDev &s, const double *misfit, float *particles_out,
                             cudaStream_t st, const double *rank)
 {
-    pso_rank_kernel<<<1, STEP_THREADS, 0, st>>>(s, misfit, rank);
+    pso_rank_kernel<<<(s.P + STEP_WARPS - 1) / STEP_WARPS + 1, STEP_THREADS, 0, st>>>(s, misfit, rank);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    // one element per thread, 256 threads a CTA (P D <= 2048 x 1024 elements)
+    // one element per thread up to four CTAs per SM of a large GPU
     const long long n = (long long)s.P * s.D;
-    const int blocks = (int)std::max<long long>(1, std::min<long long>((n + 255) / 256, 8192));
-    pso_move_kernel<<<blocks, 256, 0, st>>>(s, particles_out);
+    const int blocks = (int)std::max<long long>(1, std::min<long long>((n + STEP_THREADS - 1) / STEP_THREADS, 608));
+    pso_move_kernel<<<blocks, STEP_THREADS, 0, st>>>(s, particles_out);
+    return cudaGetLastError();
+}
+
+namespace {
+
+// the swarm's state into the caller's buffers (null ones are skipped), in one
+// launch: as six device-to-device copies it took longer than the step itself
+__global__ void state_kernel(PsoDev s, double *x, double *v, double *p, double *pf, int *order, int *gk)
+{
+    const long long n = (long long)s.P * s.D, e0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    for (long long e = e0; e < n; e += (long long)gridDim.x * blockDim.x) {
+        if (x) x[e] = s.x[e];
+        if (v) v[e] = s.v[e];
+        if (p) p[e] = s.p[e];
+    }
+    for (long long i = e0; i < s.P; i += (long long)gridDim.x * blockDim.x) {
+        if (pf) pf[i] = s.pf[i];
+        if (order) order[i] = s.order[i];
+    }
+    if (gk && e0 < 2) gk[e0] = s.gk[e0];
+}
+
+}  // namespace
+
+cudaError_t launch_pso_state(const PsoDev &s, double *x, double *v, double *p, double *pf, int *order, int *gk,
+                             cudaStream_t st)
+{
+    if (!x && !v && !p && !pf && !order && !gk) return cudaSuccess;
+    const long long n = (long long)s.P * s.D;
+    const int blocks = (int)std::max<long long>(1, std::min<long long>((n + 255) / 256, 1216));
+    state_kernel<<<blocks, 256, 0, st>>>(s, x, v, p, pf, order, gk);
     return cudaGetLastError();
 }
 
