@@ -98,6 +98,7 @@ struct empso_ctx {
     size_t stage_cap = 0;        // bytes
     cudaEvent_t stage_free = nullptr;
     int *counter = nullptr;
+    cudaMemPool_t pool = nullptr;         // stream-ordered workspace (low-pass taps)
     unsigned char *wave_ws = nullptr;     // plain streaming kernel: queue, group barriers, partial sums
     size_t wave_ws_cap = 0;               // bytes
 
@@ -899,6 +900,7 @@ void free_ctx(empso_ctx *c)
     cudaFree(c->stage_dev);
     cudaFree(c->counter);
     cudaFree(c->wave_ws);
+    if (c->pool) cudaMemPoolDestroy(c->pool);
     cudaFree(c->dev_err);
     cudaFree(c->nonfinite);
     cudaFree(c->adj.a);       // B lies inside a; G and J inside mu
@@ -1194,14 +1196,33 @@ empso_status empso_lowpass(empso_ctx *ctx, const float *in, int32_t S, int32_t n
                     "need positive sizes, finite dt_in, dt_out, f_cut, half_width > 0, in != out");
     if (((double)nt_out * dt_out + half_width) / dt_in > 1e9)
         return fail(ctx, EMPSO_INVALID_ARG, "output times beyond 1e9 input samples");
-    const long long span = lowpass_span(dt_in, dt_out, half_width);
-    const size_t smem = lowpass_smem_bytes(span);
-    if (smem > ctx->smem_optin)
+    if (!lowpass_supported(dt_in, dt_out, half_width, ctx->smem_optin))
         return fail(ctx, EMPSO_UNSUPPORTED, "filter window too long for shared memory "
                                             "(half_width / dt_in too large)");
-    CK(ctx, lowpass_configure(smem));
-    CK(ctx, launch_lowpass(in, S, nt_in, nrec, dt_in, out, nt_out, dt_out, f_cut, half_width, smem,
-                           (cudaStream_t)stream));
+    // the taps' workspace comes from the context's own pool in stream order, so
+    // that calls on several streams do not share it and a capture owns its own
+    if (!ctx->pool) {
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = ctx->device;
+        CK(ctx, cudaMemPoolCreate(&ctx->pool, &props));
+        uint64_t keep = 128ull << 20;       // bytes kept between calls
+        CK(ctx, cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep));
+    }
+    cudaStream_t st = (cudaStream_t)stream;
+    const size_t need = lowpass_ws_floats(S, nrec, nt_out, dt_in, dt_out, half_width, ctx->sm_count);
+    float *ws = nullptr;
+    const cudaError_t me = cudaMallocFromPoolAsync((void **)&ws, sizeof(float) * need, ctx->pool, st);
+    if (me == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        return fail(ctx, EMPSO_OOM, "low-pass workspace: " + std::to_string(sizeof(float) * need) + " bytes");
+    }
+    CK(ctx, me);
+    const cudaError_t e = launch_lowpass(in, S, nt_in, nrec, dt_in, out, nt_out, dt_out, f_cut, half_width, ws,
+                                         need, ctx->sm_count, st);
+    CK(ctx, cudaFreeAsync(ws, st));
+    CK(ctx, e);
     return EMPSO_OK;
 }
 

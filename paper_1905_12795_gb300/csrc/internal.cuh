@@ -155,11 +155,10 @@ cudaError_t launch_wave_l2(int R, const GridDev *grids_dev, const Inst *insts, i
                            int ring_pitch, size_t smem, double *partial, cudaStream_t st, bool hist = false);
 
 // Band-limited resampling of traces (filter.cu).
-long long lowpass_span(double dt_in, double dt_out, double W);
-size_t lowpass_smem_bytes(long long span);
-cudaError_t lowpass_configure(size_t smem);
+bool lowpass_supported(double dt_in, double dt_out, double W, size_t limit);
+size_t lowpass_ws_floats(int S, int nrec, int nt_out, double dt_in, double dt_out, double W, int sms);
 cudaError_t launch_lowpass(const float *in, int S, int nt_in, int nrec, double dt_in, float *out,
-                           int nt_out, double dt_out, double fc, double W, size_t smem,
+                           int nt_out, double dt_out, double fc, double W, float *ws, size_t ws_floats, int sms,
                            cudaStream_t st);
 
 cudaError_t launch_level_taps(const GridDev &g, int L, const float *level_z, const int *level_off,

@@ -193,7 +193,7 @@ __device__ __forceinline__ long long ordered(double f)
 // ascending sort gives it.  Every CTA keeps all keys in shared memory.  (One
 // CTA that updated every best and sorted bitonically, 55 passes over shared
 // memory for 1024 keys, took 53 us under ncu for P = 1024, D = 32; this takes
-// @RANKT@.)  The generation counter is not written here, where every CTA reads
+// 5.5.)  The generation counter is not written here, where every CTA reads
 // it: the new one goes to s.k_new for the second part, beside the constriction
 // factor (Eq. 3), whose FP64 root and quotient every thread of the second part
 // would otherwise repeat.
