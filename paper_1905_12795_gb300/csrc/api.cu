@@ -26,6 +26,9 @@ using namespace empso;
 // 9 rows 551.1)
 constexpr int RESIDENT_RUNS[] = {13, 11, 9, 8, 6};
 
+// the run lengths that the estimate of a launch's time chooses among
+constexpr int RESIDENT_RUNS_EST[] = {13, 11, 9, 8, 7, 6, 5, 4};
+
 // Occupancy answers depend only on the device and the launch shape, and the
 // planner asks for every cluster size and run length of every batch (each
 // surrogate generation plans a batch): memoised process-wide.
@@ -528,10 +531,32 @@ empso_status plan_batch(empso_ctx *ctx, const Models &mod, const empso_shot *sho
         int nrec_max = 0;
         for (int s = 0; s < S; ++s) nrec_max = std::max(nrec_max, (int)shots[s].nrec);
         const int ring_pitch = nrec_max;
+        int n_grids = 0, only = 0;
+        for (int gid = 0; gid < ng; ++gid)
+            if (p.fbase[gid] >= 0) {
+                ++n_grids;
+                only = gid;
+            }
         // every cluster size and rows-per-thread shape; the most SMs busy wins,
-        // the longer runs (fewer, fatter threads) on a tie
+        // the longer runs (fewer, fatter threads) on a tie.  A launch over one
+        // grid also estimates its time (resident_step_us) and takes the shape
+        // with the least estimate when that promises 5 % or more: the busy-SM
+        // rule ignores the rounds of instances, the halo rows and how few
+        // threads a long run leaves a small slab, and over 8 grids x 6 batch
+        // sizes was 23 % from the best shape on average (2.05 times at worst),
+        // the estimate 5 % (1.3 times).  101 x 101, order 4: one shot 384 ->
+        // 281 us, 1024 particles 10.99 -> 7.5 ms.
+        const bool est = n_grids == 1 && forcedC == 0 && forcedRows == 0;
+        double best_us = 0.0, rule_us = 0.0;
+        struct Shape {
+            int C, rows, threads, nc;
+            size_t sm;
+            std::vector<char> pair;
+        } rule{}, least{};
+        std::vector<int> runs = resident_runs(forcedRows);
+        if (est) runs.assign(std::begin(RESIDENT_RUNS_EST), std::end(RESIDENT_RUNS_EST));
         for (int C = 1; C <= 16; ++C)
-            for (const int rows : resident_runs(forcedRows)) {
+            for (const int rows : runs) {
             if (forcedC > 0 && C != forcedC) continue;
             bool ok = true;
             size_t sm = 0;
@@ -556,19 +581,38 @@ empso_status plan_batch(empso_ctx *ctx, const Models &mod, const empso_shot *sho
                                 resident_threads(g, C / 2, rows) <= threads;
                 }
             const int nc = (int)std::min<long long>(memo_resident_clusters(resR, C, threads, sm, rows), p.n_inst);
-            const long long sms = (long long)nc * C;
-            if (nc > 0 && sms > best_sms) {
-                best_sms = sms;
-                p.resident = true;
-                p.res_pair = pair;
-                p.resR = resR;
-                p.resC = C;
-                p.res_rows = rows;
-                p.res_smem = sm;
-                p.res_threads = threads;
-                p.res_clusters = nc;
-                p.ring_pitch = ring_pitch;
+            if (nc <= 0) continue;
+            double us = 0.0;
+            if (est) {
+                us = (double)((p.n_inst + nc - 1) / nc) *
+                     resident_step_us(ctx->grids[only].dev, C, rows, threads, std::max(1.0, (double)nc * C / ctx->sm_count));
+                // (one receiver per thread at most: the FP32 partial sums of a
+                // misfit then do not depend on the shape)
+                if ((nrec_max + C - 1) / C <= threads && (!least.C || us < best_us)) {
+                    best_us = us;
+                    least = {C, rows, threads, nc, sm, pair};
+                }
+                if (std::find(std::begin(RESIDENT_RUNS), std::end(RESIDENT_RUNS), rows) == std::end(RESIDENT_RUNS))
+                    continue;
             }
+            const long long sms = (long long)nc * C;
+            if (sms > best_sms) {
+                best_sms = sms;
+                rule_us = us;
+                rule = {C, rows, threads, nc, sm, pair};
+            }
+        }
+        const Shape &shape = least.C && (!rule.C || best_us * 1.05 < rule_us) ? least : rule;
+        if (shape.C) {
+            p.resident = true;
+            p.res_pair = shape.pair;
+            p.resR = resR;
+            p.resC = shape.C;
+            p.res_rows = shape.rows;
+            p.res_smem = shape.sm;
+            p.res_threads = shape.threads;
+            p.res_clusters = shape.nc;
+            p.ring_pitch = ring_pitch;
         }
     }
     if (kind == EMPSO_KERNEL_RESIDENT && !p.resident)

@@ -202,6 +202,7 @@ int resident_default_rows();
 bool resident_rows_supported(int rows);
 int resident_grid_run(const GridDev &g, int Ce, int threads, int rows);
 int resident_threads(const GridDev &g, int C, int rows);
+double resident_step_us(const GridDev &g, int C, int rows, int threads, double k);
 size_t resident_smem_bytes(const GridDev &g, int C, int ring_pitch);
 bool resident_fits(const GridDev &g, int C, int ring_pitch, size_t smem_limit, int rows);
 cudaError_t resident_configure(int R, size_t smem_bytes, int C);

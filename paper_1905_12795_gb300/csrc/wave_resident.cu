@@ -24,6 +24,8 @@
 // batch by the planner and the autotuner.
 #include <cooperative_groups.h>
 
+#include <algorithm>
+
 #include "internal.cuh"
 #include "stencil.cuh"
 
@@ -661,6 +663,25 @@ bool resident_fits(const GridDev &g, int C, int ring_pitch, size_t smem_limit, i
     }
     if (resident_threads(g, C, rows) > shape_threads(rows)) return false;
     return resident_smem_bytes(g, C, ring_pitch) <= smem_limit;
+}
+
+// Estimated time of one step, in microseconds, of grid g on clusters of C CTAs
+// of `threads` threads with runs of at most `rows` rows, k CTAs to an SM: the
+// barrier, the rows a thread sweeps one after the other (extra single rows at
+// EXTRA rows each: they load a whole window), and the work of the CTAs that
+// share an SM.  The constants are a fit to 3759 launches (8 grids of order 2, 4
+// and 8, 1 to 1024 instances, every cluster size, runs of 4 to 13 rows; 10 % rms
+// over the shapes within 1.5 of the best).
+double resident_step_us(const GridDev &g, int C, int rows, int threads, double k)
+{
+    constexpr double BARRIER = 1.089, PER_CTA = 0.0025, EXTRA = 6.88, LAT = 0.0339, LAT_R = 0.0043, WORK = 0.0019,
+                     WORK_R = 0.0084, WARPS = 0.0906, CARRIED = 0.11;
+    const int rows_c = (g.NZ + C - 1) / C, nseg = (rows_c + rows - 1) / rows, run = (rows_c + nseg - 1) / nseg;
+    const int left = std::max(0, g.NQ * nseg - threads);
+    double q = run + EXTRA * left * run / threads;
+    if (rows > RW_A && g.R == 4) q *= 1.0 - CARRIED;     // the shape that carries its z-differences
+    const double per = (threads / 32 + 3) / 4;           // warps of a scheduler
+    return BARRIER + PER_CTA * C + (LAT + LAT_R * g.R) * q + k * per * ((WORK + WORK_R * g.R) * q + WARPS);
 }
 
 // Rows per run for grid g in a launch of `threads` threads with runs of at
