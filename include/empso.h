@@ -201,9 +201,10 @@ empso_status empso_generation(empso_ctx *ctx, const empso_shot *shots, int32_t S
                               const float *d_obs, double *misfit_out, void *stream);
 
 /* Autotuner: times the streaming kernel, the on-chip kernel at every cluster
- * size and rows-per-thread shape the batch fits, and the L2 cluster kernel at
- * cluster sizes 4, 8, 10, 12 and 16 (one warm-up and one timed launch each,
- * CUDA events on `stream`) on this exact batch (particles device [P][K],
+ * size and rows-per-thread shape the batch fits, and the L2 kernel on its
+ * own split of the GPU (cluster 0) and on 4, 8, 10, 12 and 16 SMs per
+ * instance (one warm-up and one timed launch each, CUDA events on `stream`) on
+ * this exact batch (particles device [P][K],
  * shots, d_obs; misfit device [P] is used as scratch output), and keeps the
  * fastest for every later batch with the same grids, shot counts and P.  With
  * a kernel kind selected (empso_set_kernel), only that kind's candidates are
@@ -322,10 +323,10 @@ empso_status surrogate_generation(empso_ctx *ctx, const empso_shot *shots, int32
  *   EMPSO_KERNEL_RESIDENT   wavefields in distributed shared memory, one
  *                           thread-block cluster per instance (calls return
  *                           UNSUPPORTED when a grid does not fit);
- *   EMPSO_KERNEL_CLUSTER_L2 wavefields in a per-cluster global buffer, one
- *                           thread-block cluster per instance, with few
- *                           enough instances in flight to stay in L2 (for
- *                           grids too large for the on-chip variant).
+ *   EMPSO_KERNEL_CLUSTER_L2 wavefields in global memory, a group of
+ *                           co-resident CTAs per instance, with few enough
+ *                           instances in flight to stay in L2 (for grids
+ *                           too large for the on-chip variant).
  * All compute the same scheme; results agree to FP32 rounding. */
 #define EMPSO_KERNEL_AUTO      0
 #define EMPSO_KERNEL_STREAMING 1
@@ -333,8 +334,8 @@ empso_status surrogate_generation(empso_ctx *ctx, const empso_shot *shots, int32
 #define EMPSO_KERNEL_CLUSTER_L2 3
 empso_status empso_set_kernel(empso_ctx *ctx, int32_t kind);
 
-/* Cluster size (CTAs per instance) of the on-chip kernel: 0 lets the library
- * pick the size that keeps the most SMs busy; 1..16 forces it (calls return
+/* Cluster size (CTAs per instance) of the on-chip kernel, SMs per instance of
+ * the L2 kernel: 0 lets the library pick it; 1..16 forces it (calls return
  * UNSUPPORTED when the batch does not fit that size). */
 empso_status empso_set_cluster(empso_ctx *ctx, int32_t ctas);
 

@@ -47,21 +47,6 @@ int memo_resident_clusters(int R, int C, int threads, size_t smem, int rows, boo
     return n;
 }
 
-int memo_l2_clusters(int R, int C, int threads, size_t smem, bool hist = false)
-{
-    static std::mutex mu;
-    static std::map<std::tuple<int, int, int, int, size_t, bool>, int> memo;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const auto key = std::make_tuple(dev, R, C, threads, smem, hist);
-    std::lock_guard<std::mutex> lock(mu);
-    const auto it = memo.find(key);
-    if (it != memo.end()) return it->second;
-    const int n = l2_max_clusters(R, C, threads, smem, hist);
-    if (n >= 0) memo[key] = n;       // errors (negative) are not kept
-    return n;
-}
-
 // the run lengths to consider: the forced one, else RESIDENT_RUNS
 std::vector<int> resident_runs(int forced)
 {
@@ -448,10 +433,8 @@ struct Plan {
     int n_units = 0, n_paired = 0;
     int n_ctas = 0;
     bool l2 = false;                   // L2-resident cluster kernel
-    int l2C = 0, l2_clusters = 0, l2_threads = 0;
-    long long l2_slot_f4 = 0;
-    size_t l2_smem = 0;
-    WaveSplit wave{};                  // plain streaming kernel: instances in flight, CTAs for each
+    int l2C = 0;
+    WaveSplit wave{};                  // L2 and plain streaming kernels: instances in flight, CTAs for each
     int wave_R = 0;                    // its stencil radius (0: the grids differ)
     bool stream_tma = false;           // streaming path: row-pipelined bulk-copy kernel
     int st_threads = 0, st_R = 0, rec_max = 0;
@@ -540,7 +523,8 @@ empso_status plan_batch(empso_ctx *ctx, const Models &mod, const empso_shot *sho
         // every cluster size and rows-per-thread shape; the most SMs busy wins,
         // the longer runs (fewer, fatter threads) on a tie.  A launch over one
         // grid also estimates its time (resident_step_us) and takes the shape
-        // with the least estimate when that promises 5 % or more: the busy-SM
+        // with the least estimate when that promises 5 % or more (15 % at order 2,
+        // where the estimate is rougher): the busy-SM
         // rule ignores the rounds of instances, the halo rows and how few
         // threads a long run leaves a small slab, and over 8 grids x 6 batch
         // sizes was 23 % from the best shape on average (2.05 times at worst),
@@ -602,7 +586,7 @@ empso_status plan_batch(empso_ctx *ctx, const Models &mod, const empso_shot *sho
                 rule = {C, rows, threads, nc, sm, pair};
             }
         }
-        const Shape &shape = least.C && (!rule.C || best_us * 1.05 < rule_us) ? least : rule;
+        const Shape &shape = least.C && (!rule.C || best_us * (resR == 1 ? 1.15 : 1.05) < rule_us) ? least : rule;
         if (shape.C) {
             p.resident = true;
             p.res_pair = shape.pair;
@@ -626,50 +610,30 @@ empso_status plan_batch(empso_ctx *ctx, const Models &mod, const empso_shot *sho
             if (p.fbase[gid] >= 0)
                 p.res_run[gid] = resident_grid_run(ctx->grids[gid].dev, p.res_pair[gid] ? p.resC / 2 : p.resC,
                                                    p.res_threads, p.res_rows);
-    // L2-resident cluster kernel for grids the on-chip kernel cannot hold:
-    // the cluster size that keeps the most SMs busy while every instance in
-    // flight (two time levels and the model field) stays within the L2 budget
+    // L2 kernel for grids the on-chip kernel cannot hold: the split of the GPU
+    // with the least estimated time while every instance in flight (two time
+    // levels and the model field) stays within the L2 budget
     p.l2 = false;
     if (!p.resident && resR > 0 && (kind == EMPSO_KERNEL_AUTO || kind == EMPSO_KERNEL_CLUSTER_L2)) {
         int nrec_max = 0;
         for (int s = 0; s < S; ++s) nrec_max = std::max(nrec_max, (int)shots[s].nrec);
-        const size_t sm = l2_smem_bytes(nrec_max);
-        long long best_sms = 0;
-        for (int C : {16, 12, 10, 8, 6, 4, 3, 2, 1}) {
-            if (forcedC > 0 && C != forcedC) continue;
-            bool ok = sm <= ctx->smem_optin;
-            long long slot = 0, inst_bytes = 0, items = 32;
-            for (int gid = 0; gid < ng && ok; ++gid) {
-                if (p.fbase[gid] < 0) continue;
-                const GridDev &g = ctx->grids[gid].dev;
-                ok = l2_fits(g, C);
-                slot = std::max(slot, l2_slot_f4(g, C));
-                inst_bytes = std::max(inst_bytes, 32 * l2_slot_f4(g, C) + 4 * g.field);
-                const int rows_c = (g.NZ + C - 1) / C;
-                items = std::max<long long>(items, (long long)g.NQ * ((rows_c + 7) / 8));
-            }
-            if (!ok) continue;
-            const int threads = (int)std::min<long long>(l2_max_threads(), (items + 31) / 32 * 32);
-            CK(ctx, l2_configure(resR, sm, C));
-            const long long by_l2 = std::max<long long>(1, L2_BUDGET_BYTES / std::max<long long>(inst_bytes, 1));
-            const int occ = memo_l2_clusters(resR, C, threads, sm);
-            if (occ < 0)
-                return fail(ctx, EMPSO_CUDA_ERROR,
-                            std::string("L2 cluster kernel occupancy (C = ") + std::to_string(C) +
-                                "): " + cudaGetErrorString((cudaError_t)(-occ)));
-            const int nc = (int)std::min<long long>(std::min<long long>(occ, p.n_inst), by_l2);
-            const long long sms = (long long)nc * C;
-            if (nc > 0 && sms > best_sms) {
-                best_sms = sms;
-                p.l2 = true;
-                p.resR = resR;
-                p.l2C = C;
-                p.l2_clusters = nc;
-                p.l2_threads = threads;
-                p.l2_slot_f4 = slot;
-                p.l2_smem = sm;
-                p.ring_pitch = nrec_max;
-            }
+        std::vector<const GridDev *> used;
+        bool ok = true;
+        long long inst_bytes = 1;
+        for (int gid = 0; gid < ng; ++gid) {
+            if (p.fbase[gid] < 0) continue;
+            const GridDev &g = ctx->grids[gid].dev;
+            used.push_back(&g);
+            ok = ok && l2_fits(g, std::max(1, forcedC), nrec_max, ctx->smem_optin);
+            inst_bytes = std::max(inst_bytes, 12 * g.field);
+        }
+        if (ok) {
+            p.wave = l2_split(used.data(), (int)used.size(), resR, p.n_inst, L2_BUDGET_BYTES / inst_bytes, forcedC,
+                              ctx->sm_count);
+            if (p.wave.group < 1) return fail(ctx, EMPSO_CUDA_ERROR, "occupancy of the L2 kernel");
+            p.l2 = true;
+            p.resR = resR;
+            p.l2C = forcedC > 0 ? forcedC : p.wave.group;
         }
     }
     if (kind == EMPSO_KERNEL_CLUSTER_L2 && !p.l2)
@@ -708,6 +672,8 @@ empso_status plan_batch(empso_ctx *ctx, const Models &mod, const empso_shot *sho
         }
         p.wave = wave_split(used.data(), (int)used.size(), p.wave_R, p.n_inst, L2_BUDGET_BYTES / inst_bytes);
         if (p.wave.group < 1) return fail(ctx, EMPSO_CUDA_ERROR, "occupancy of the streaming kernel");
+    }
+    if (!p.resident && !p.stream_tma) {
         // sized once, for any split of this device (captured generations keep the pointer)
         if ((rc = grow(ctx, (void **)&ctx->wave_ws, &ctx->wave_ws_cap, wave_ws_bytes(), 1)) != EMPSO_OK) return rc;
         max_ctas = p.wave.flight;
@@ -716,11 +682,7 @@ empso_status plan_batch(empso_ctx *ctx, const Models &mod, const empso_shot *sho
     if ((rc = grow(ctx, (void **)&ctx->fields, &ctx->fields_cap, sizeof(float) * ftotal,
                    sizeof(float))) != EMPSO_OK)
         return rc;
-    if (p.l2 &&
-        (rc = grow(ctx, (void **)&ctx->slots, &ctx->slots_cap,
-                   sizeof(float4) * 2 * (size_t)p.l2_slot_f4 * p.l2_clusters, sizeof(float))) != EMPSO_OK)
-        return rc;
-    if (!p.resident && !p.l2 &&
+    if (!p.resident &&
         (rc = grow(ctx, (void **)&ctx->slots, &ctx->slots_cap,
                    sizeof(float) * 2 * p.maxfield * p.n_ctas, sizeof(float))) != EMPSO_OK)
         return rc;
@@ -840,13 +802,11 @@ empso_status enqueue_batch(empso_ctx *ctx, const Models &mod, const Plan &p, dou
         ctx->last_groups = p.res_clusters;
         ctx->last_paired = p.n_paired;
     } else if (p.l2) {
-        CK(ctx, launch_wave_l2(p.resR, ctx->grids_dev, p.insts,
-                               (int)p.n_inst, ctx->counter, p.l2C, p.l2_clusters, p.l2_threads,
-                               reinterpret_cast<float4 *>(ctx->slots), p.l2_slot_f4, p.ring_pitch,
-                               p.l2_smem, ctx->partial, st));
+        CK(ctx, launch_wave_l2(p.resR, ctx->grids_dev, p.insts, (int)p.n_inst, p.wave, ctx->wave_ws, ctx->slots,
+                               2 * p.maxfield, ctx->dev_err, ctx->partial, st));
         ctx->last_path = 4;
         ctx->last_C = p.l2C;
-        ctx->last_groups = p.l2_clusters;
+        ctx->last_groups = p.wave.flight;
     } else if (p.stream_tma) {
         CK(ctx, launch_wave_stream(p.st_R, ctx->grids_dev, p.insts, (int)p.n_inst, ctx->counter,
                                    ctx->slots, 2 * p.maxfield, p.n_ctas, p.st_threads, p.st_smem,
@@ -1376,57 +1336,29 @@ empso_status gradient_impl(empso_ctx *ctx, const float *vel, int M, const empso_
     }
     if (ctx->kernel_kind == EMPSO_KERNEL_RESIDENT && !rC)
         return fail(ctx, EMPSO_UNSUPPORTED, "gradient: the grid does not fit the on-chip kernel");
-    // else the L2 cluster kernel, also streaming the history out, when the
-    // selection allows it and the grid fits: the cluster size that keeps the
-    // most SMs busy with the instances in flight inside the L2 budget
-    int lC = 0, l_threads = 0, l_nc = 0;
-    long long l_slot = 0;
-    size_t l_smem = 0;
-    if (!rC && g.R <= MAX_R_FAST &&
-        (ctx->kernel_kind == EMPSO_KERNEL_AUTO || ctx->kernel_kind == EMPSO_KERNEL_CLUSTER_L2)) {
-        const size_t sm = l2_smem_bytes(rec_max);
-        long long best = 0;
-        for (int C : {16, 12, 10, 8, 6, 4, 3, 2, 1}) {
-            if (sm > ctx->smem_optin || !l2_fits(g, C)) continue;
-            const long long slot = l2_slot_f4(g, C);
-            const long long inst_bytes = 32 * slot + 4 * g.field;
-            const int rows_c = (g.NZ + C - 1) / C;
-            const long long items = std::max<long long>(32, (long long)g.NQ * ((rows_c + 7) / 8));
-            const int threads = (int)std::min<long long>(l2_max_threads(), (items + 31) / 32 * 32);
-            CK(ctx, l2_configure(g.R, sm, C));
-            const int occ = memo_l2_clusters(g.R, C, threads, sm, true);
-            if (occ <= 0) continue;
-            const long long by_l2 = std::max<long long>(1, L2_BUDGET_BYTES / inst_bytes);
-            const int nc = (int)std::min<long long>(std::min<long long>(occ, I), by_l2);
-            if ((long long)nc * C > best) {
-                best = (long long)nc * C;
-                lC = C;
-                l_threads = threads;
-                l_nc = nc;
-                l_slot = slot;
-                l_smem = sm;
-            }
-        }
-    }
-    if (ctx->kernel_kind == EMPSO_KERNEL_CLUSTER_L2 && !lC)
-        return fail(ctx, EMPSO_UNSUPPORTED, "gradient: the grid does not fit the L2 cluster kernel");
-    // the cluster kernels hold stencils up to radius 4; order 16 runs its forward
-    // pass on the plain streaming kernel, which streams the history out too
+    // else the L2 kernel, or for order 16 the plain streaming kernel, also
+    // streaming the history out, when the selection allows it and the grid fits
     WaveSplit split{};
-    if (g.R > MAX_R_FAST) {
-        const GridDev *gp = &g;
-        split = wave_split(&gp, 1, g.R, I, L2_BUDGET_BYTES / (12 * g.field), true);
-        if (split.group < 1) return fail(ctx, EMPSO_CUDA_ERROR, "gradient: occupancy of the streaming kernel");
+    const GridDev *gp = &g;
+    const long long by_l2 = L2_BUDGET_BYTES / (12 * g.field);
+    const bool l2 = !rC && g.R <= MAX_R_FAST && l2_fits(g, 1, rec_max, ctx->smem_optin) &&
+                    (ctx->kernel_kind == EMPSO_KERNEL_AUTO || ctx->kernel_kind == EMPSO_KERNEL_CLUSTER_L2);
+    if (ctx->kernel_kind == EMPSO_KERNEL_CLUSTER_L2 && !l2)
+        return fail(ctx, EMPSO_UNSUPPORTED, "gradient: the grid does not fit the L2 cluster kernel");
+    if (l2) split = l2_split(&gp, 1, g.R, I, by_l2, 0, ctx->sm_count, true);
+    if (g.R > MAX_R_FAST) split = wave_split(&gp, 1, g.R, I, by_l2, true);
+    if ((l2 || g.R > MAX_R_FAST) && split.group < 1)
+        return fail(ctx, EMPSO_CUDA_ERROR, "gradient: occupancy of the forward kernel");
+    if (split.group) {
         if ((rc = adj_grow(ctx, &W.wave_ws, &W.wave_ws_cap, wave_ws_bytes(), nullptr))) return rc;
         if ((rc = adj_grow(ctx, &W.slots, &W.slots_cap, F / 2 * split.flight, nullptr))) return rc;
     }
     const size_t r_ofs = ((size_t)I * sizeof(Inst) + 255) / 256 * 256;
-    const bool table = rC || lC || split.group;
+    const bool table = rC || split.group;
     if (table) {
         if ((rc = adj_grow(ctx, &W.rtab, &W.rtab_cap, r_ofs + sizeof(int4) * (size_t)I, nullptr))) return rc;
         if ((rc = adj_grow(ctx, &W.counter, &W.counter_cap, 1, nullptr))) return rc;
     }
-    if (lC && (rc = adj_grow(ctx, &W.slots, &W.slots_cap, 2 * (size_t)l_slot * l_nc, nullptr))) return rc;
     // instance tables (the previous call's kernels may still read the old ones)
     std::vector<AdjInst> hi((size_t)I);
     std::vector<unsigned char> rh(table ? r_ofs + sizeof(int4) * (size_t)I : 0);
@@ -1481,7 +1413,7 @@ empso_status gradient_impl(empso_ctx *ctx, const float *vel, int M, const empso_
     CK(ctx, launch_adj_prep(g, W.a, W.B, M, st));
     // the two time loops replay as one graph
     std::ostringstream key;
-    key << gid << "|" << I << "|" << rec_threads << "|" << (const void *)W.insts << "|" << rC << "|" << lC
+    key << gid << "|" << I << "|" << rec_threads << "|" << (const void *)W.insts << "|" << rC << "|" << split.group
         << "|" << (const void *)W.rtab << "|" << (const void *)W.slots << "|" << forward_only << "|"
         << ctx->grad_chains;
     cudaGraphExec_t exec = nullptr;
@@ -1499,17 +1431,12 @@ empso_status gradient_impl(empso_ctx *ctx, const float *vel, int M, const empso_
                                           W.counter, rC, r_nc, r_threads, r_rows, rec_max, r_smem, W.phi,
                                           ctx->cap_stream, true);
             if (ce == cudaSuccess) ce = launch_adj_residual(g, W.insts, (int)I, rec_max, ctx->cap_stream);
-        } else if (lC) {
-            ce = cudaMemsetAsync(W.counter, 0, sizeof(int), ctx->cap_stream);
-            if (ce == cudaSuccess)
-                ce = launch_wave_l2(g.R, ctx->grids_dev, reinterpret_cast<const Inst *>(W.rtab), (int)I, W.counter,
-                                    lC, l_nc, l_threads, W.slots, l_slot, rec_max, l_smem, W.phi,
-                                    ctx->cap_stream, true);
-            if (ce == cudaSuccess) ce = launch_adj_residual(g, W.insts, (int)I, rec_max, ctx->cap_stream);
         } else if (split.group) {
-            ce = launch_wave(g.R, ctx->grids_dev, reinterpret_cast<const Inst *>(W.rtab), (int)I, split, W.wave_ws,
-                             reinterpret_cast<float *>(W.slots), 2 * g.field, ctx->dev_err, W.phi, ctx->cap_stream,
-                             !forward_only);
+            // (the misfit alone: no history)
+            const auto launch = l2 ? launch_wave_l2 : launch_wave;
+            ce = launch(g.R, ctx->grids_dev, reinterpret_cast<const Inst *>(W.rtab), (int)I, split, W.wave_ws,
+                        reinterpret_cast<float *>(W.slots), 2 * g.field, ctx->dev_err, W.phi, ctx->cap_stream,
+                        !forward_only);
             if (ce == cudaSuccess) ce = launch_adj_residual(g, W.insts, (int)I, rec_max, ctx->cap_stream);
         } else {
             // the per-step forward pass with its time levels in the (zeroed)
@@ -1981,7 +1908,7 @@ empso_status empso_autotune(empso_ctx *ctx, const float *particles, int32_t P,
         for (int C = 1; C <= 16; ++C)
             for (const int rows : RESIDENT_RUNS) cand.push_back({EMPSO_KERNEL_RESIDENT, C, rows});
     if (only == EMPSO_KERNEL_AUTO || only == EMPSO_KERNEL_CLUSTER_L2)
-        for (int C : {4, 8, 10, 12, 16}) cand.push_back({EMPSO_KERNEL_CLUSTER_L2, C, 0});
+        for (int C : {0, 4, 8, 10, 12, 16}) cand.push_back({EMPSO_KERNEL_CLUSTER_L2, C, 0});   // 0: the planner's split
     float best = 1e30f;
     empso_ctx::Tuned choice;
     choice.kind = EMPSO_KERNEL_AUTO;
@@ -2007,7 +1934,7 @@ empso_status empso_autotune(empso_ctx *ctx, const float *particles, int32_t P,
         if (ms < best) {
             best = ms;
             choice.kind = c.kind;
-            choice.C = p.resident ? p.resC : (p.l2 ? p.l2C : 0);
+            choice.C = p.resident ? p.resC : (p.l2 ? c.C : 0);
             choice.rows = p.resident ? p.res_rows : 0;
         }
     }

@@ -140,20 +140,6 @@ cudaError_t launch_fwi_step(const float *v, const float *g, float alpha, float v
 cudaError_t launch_fwi_dots(const float *a, const float *b, const float *c, const float *d, int n,
                             double *r, cudaStream_t st);
 
-// L2-resident cluster variant (wave_l2.cu): time levels in a per-cluster
-// global buffer of l2_slot_f4 float4 each.
-int l2_max_threads();
-size_t l2_smem_bytes(int ring_pitch);
-long long l2_slot_f4(const GridDev &g, int C);
-bool l2_fits(const GridDev &g, int C);
-cudaError_t l2_configure(int R, size_t smem, int C);
-// clusters of the modelling (hist = false) or history (hist = true) instantiation
-// that fit the device at once
-int l2_max_clusters(int R, int C, int threads, size_t smem, bool hist = false);
-cudaError_t launch_wave_l2(int R, const GridDev *grids_dev, const Inst *insts, int n_inst, int *counter,
-                           int C, int n_clusters, int threads, float4 *slots, long long slot_f4,
-                           int ring_pitch, size_t smem, double *partial, cudaStream_t st, bool hist = false);
-
 // Band-limited resampling of traces (filter.cu).
 bool lowpass_supported(double dt_in, double dt_out, double W, size_t limit);
 size_t lowpass_ws_floats(int S, int nrec, int nt_out, double dt_in, double dt_out, double W, int sms);
@@ -175,13 +161,23 @@ constexpr int WAVE_MAX_CTAS = 4096;      // co-resident CTAs of any device
 struct WaveSplit {
     int flight, group;
 };
-int wave_max_ctas(int R, bool hist = false);
 WaveSplit wave_split(const GridDev *const *grids, int n_grids, int R, long long n_inst, long long by_l2,
                      bool hist = false);
-constexpr size_t wave_ws_bytes(int flight = WAVE_MAX_CTAS) { return 128 * (1 + (size_t)flight) + sizeof(double) * WAVE_MAX_CTAS; }
+constexpr size_t wave_ws_bytes(int flight = WAVE_MAX_CTAS)
+{
+    return 128 * (1 + (size_t)flight) + sizeof(double) * WAVE_MAX_CTAS;
+}
 cudaError_t launch_wave(int R, const GridDev *grids_dev, const Inst *insts, int n_inst, const WaveSplit &s,
                         void *ws, float *slots, long long slot_floats, int *err, double *partial,
                         cudaStream_t st, bool hist = false);
+// L2-resident variant (wave_l2.cu), on the same groups and workspace (radius up
+// to 4).
+bool l2_fits(const GridDev &g, int C, int nrec, size_t limit);
+WaveSplit l2_split(const GridDev *const *grids, int n_grids, int R, long long n_inst, long long by_l2, int C, int sms,
+                   bool hist = false);
+cudaError_t launch_wave_l2(int R, const GridDev *grids_dev, const Inst *insts, int n_inst, const WaveSplit &s,
+                           void *ws, float *slots, long long slot_floats, int *err, double *partial,
+                           cudaStream_t st, bool hist = false);
 cudaError_t launch_finalize(const double *partial, const float *weights, int P, int S,
                             double *misfit, unsigned long long *nf, cudaStream_t st);
 
