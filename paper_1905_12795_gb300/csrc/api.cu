@@ -2145,6 +2145,7 @@ empso_status surrogate_init(empso_ctx *ctx, int32_t hidden, int32_t capacity, fl
     CK(ctx, alloc((void **)&s.tb, 4 * R));
     CK(ctx, alloc((void **)&s.loss, 4));
     CK(ctx, alloc((void **)&s.stats, 8));
+    CK(ctx, alloc((void **)&s.tiles, sur_tile_bytes(K, H) * ((R + 127) / 128)));
     CK(ctx, alloc((void **)&s.xbuf, 4 * (size_t)capacity * K));
     CK(ctx, alloc((void **)&s.ybuf, 4 * (size_t)capacity));
     CK(ctx, alloc((void **)&s.count, 4));
@@ -2171,7 +2172,7 @@ empso_status surrogate_init(empso_ctx *ctx, int32_t hidden, int32_t capacity, fl
     CK(ctx, cudaMemset(s.rho, 0, 4));
     CK(ctx, cudaMemcpy(s.stats, stats0, 8, cudaMemcpyHostToDevice));
     CK(ctx, sur_refresh_bf16(s, 0));
-    CK(ctx, sur_prepare_tc());
+    CK(ctx, sur_prepare_tc(s));
     s.tc = 1;
     s.err = ctx->dev_err;
     CK(ctx, cudaStreamCreateWithFlags(&ctx->sur_stream, cudaStreamNonBlocking));
@@ -2292,8 +2293,7 @@ empso_status surrogate_grad(empso_ctx *ctx, const float *particles, const float 
         return fail(ctx, EMPSO_INVALID_ARG, "bad particles/target/grad");
     cudaStream_t st = (cudaStream_t)stream;
     SurDev &s = ctx->sur;
-    CK(ctx, sur_normalize(s, particles, n, s.Xb, st));
-    CK(ctx, sur_backward(s, s.Xb, target, n, loss ? loss : s.loss, st));
+    CK(ctx, sur_gradient(s, particles, target, n, loss ? loss : s.loss, st));
     CK(ctx, cudaMemcpyAsync(grad, s.g, 4 * (size_t)s.n_params, cudaMemcpyDeviceToDevice, st));
     return EMPSO_OK;
 }

@@ -256,6 +256,7 @@ struct SurDev {
     __nv_bfloat16 *Xb = nullptr, *A1b = nullptr, *dZb = nullptr, *dZ1b = nullptr;
     float *Z2 = nullptr, *y = nullptr, *dy = nullptr, *dZf = nullptr, *dA = nullptr;
     float *tb = nullptr, *loss = nullptr, *stats = nullptr;
+    unsigned char *tiles = nullptr;   // the whole-network kernels' batch tiles and partial sums
     float *xbuf = nullptr, *ybuf = nullptr;
     int *count = nullptr;
     uint64_t seed = 0;
@@ -269,6 +270,7 @@ struct SurDev {
 };
 cudaError_t sur_backward(const SurDev &s, const __nv_bfloat16 *Xb, const float *t, int n, float *loss,
                          cudaStream_t st);
+cudaError_t sur_gradient(const SurDev &s, const float *x, const float *t, int n, float *loss, cudaStream_t st);
 cudaError_t sur_adam(SurDev &s, cudaStream_t st);
 cudaError_t sur_refresh_bf16(const SurDev &s, cudaStream_t st);
 cudaError_t sur_normalize(const SurDev &s, const float *x, int n, __nv_bfloat16 *out, cudaStream_t st);
@@ -283,7 +285,9 @@ cudaError_t sur_select(const float *key, int P, int k, int *rows, cudaStream_t s
 // logphi[rows[j]] (their predictions) into *rho (one block)
 cudaError_t sur_rank_corr(const double *fk, const int *rows, const float *logphi, int k, float *rho,
                           cudaStream_t st);
-cudaError_t sur_prepare_tc();
+cudaError_t sur_prepare_tc(const SurDev &s);
+bool sur_whole(const SurDev &s);
+size_t sur_tile_bytes(int K, int H);
 cudaError_t sur_gather(const float *x, const int *rows, int k, int K, float *out, cudaStream_t st);
 cudaError_t sur_scatter(const int *rows, const double *fk, int k, const float *logphi, int P,
                         double *fit, double *rank, cudaStream_t st);

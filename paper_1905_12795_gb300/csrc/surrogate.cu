@@ -5,6 +5,7 @@
 // (BF16 operands, FP32 accumulation), master weights and Adam moments are
 // FP32, and the training set is a device-side replay buffer filled with the
 // (particle, misfit) pairs the fitness evaluation produces.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
 #include "internal.cuh"
@@ -614,20 +615,28 @@ __global__ void head_kernel(const float *__restrict__ Z2, int n, int H, const fl
     }
 }
 
-// Adam on FP32 master weights, then BF16 copies of the two hidden matrices
-__global__ void adam_kernel(float *p, const float *__restrict__ g, float *m, float *v, long long n,
-                            float lr, float b1, float b2, float eps, float c1, float c2,
+// Adam on FP32 master weights
+struct AdamStep {
+    float lr, b1, b2, eps, c1, c2;
+    __device__ __forceinline__ float operator()(float w, float gi, float &m, float &v) const
+    {
+        m = b1 * m + (1.f - b1) * gi;
+        v = b2 * v + (1.f - b2) * gi * gi;
+        return w - lr * (m / c1) / (sqrtf(v / c2) + eps);
+    }
+};
+
+// all parameters, then BF16 copies of the two hidden matrices
+__global__ void adam_kernel(float *p, const float *__restrict__ g, float *m, float *v, long long n, AdamStep step,
                             __nv_bfloat16 *w1b, long long n_w1, __nv_bfloat16 *w2b, long long off_w2,
                             long long n_w2)
 {
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
          e += (long long)gridDim.x * blockDim.x) {
-        const float gi = g[e];
-        const float mi = b1 * m[e] + (1.f - b1) * gi;
-        const float vi = b2 * v[e] + (1.f - b2) * gi * gi;
+        float mi = m[e], vi = v[e];
+        const float w = step(p[e], g[e], mi, vi);
         m[e] = mi;
         v[e] = vi;
-        const float w = p[e] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
         p[e] = w;
         if (e < n_w1) w1b[e] = __float2bfloat16(w);
         else if (e >= off_w2 && e < off_w2 + n_w2) w2b[e - off_w2] = __float2bfloat16(w);
@@ -657,12 +666,26 @@ __device__ __forceinline__ uint4 philox_s(uint4 c, uint32_t k0, uint32_t k1)
     return c;
 }
 
-// A minibatch, one warp per row: the row drawn uniformly from the filled part of
-// the replay buffer (its first min(have_host, cap) rows when have_host >= 0,
-// else the device count's; with recent > 0 the second half of the batch comes
-// from the newest min(recent, filled) pairs instead, the swarm's current
-// neighbourhood), its standardised target (log phi - mu) / sigma and its
-// position scaled to [-1, 1] in BF16 (the buffer holds raw positions).
+// Row b of a minibatch of B: drawn uniformly from the filled part of the replay
+// buffer (`total` pairs appended so far, `cap` kept); with recent > 0 the second
+// half of the batch comes from the newest min(recent, filled) pairs instead (the
+// swarm's current neighbourhood).
+__device__ __forceinline__ int batch_row(int b, int B, int total, int cap, uint64_t seed, int step, int recent)
+{
+    const int have = min(total, cap);
+    const uint4 w = philox_s(make_uint4((uint32_t)step, (uint32_t)b, 0x5u, 0x7u), (uint32_t)seed,
+                             (uint32_t)(seed >> 32));
+    if (recent > 0 && b >= B / 2 && have > 0) {
+        const int span = min(recent, have);
+        const int j = (int)(((unsigned long long)w.x * (unsigned long long)span) >> 32);
+        return (int)(((long long)total - 1 - j) % cap);
+    }
+    return have > 0 ? (int)(((unsigned long long)w.x * (unsigned long long)have) >> 32) : 0;
+}
+
+// A minibatch, one warp per row: the drawn row's standardised target (log phi -
+// mu) / sigma and its position scaled to [-1, 1] in BF16 (the buffer, of which
+// have_host >= 0 pairs are used, else the device's count, holds raw positions).
 __global__ void batch_kernel(int B, int K, const int *count, int have_host, int cap, uint64_t seed, int step,
                              int recent, const float *__restrict__ xbuf, const float *__restrict__ ybuf,
                              const float *__restrict__ stats, const double *__restrict__ xmin,
@@ -670,18 +693,7 @@ __global__ void batch_kernel(int B, int K, const int *count, int have_host, int 
 {
     const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (b >= B) return;
-    const int total = have_host >= 0 ? have_host : *count;   // pairs appended so far
-    const int have = min(total, cap);
-    const uint4 w = philox_s(make_uint4((uint32_t)step, (uint32_t)b, 0x5u, 0x7u), (uint32_t)seed,
-                             (uint32_t)(seed >> 32));
-    int row;
-    if (recent > 0 && b >= B / 2 && have > 0) {
-        const int span = min(recent, have);
-        const int j = (int)(((unsigned long long)w.x * (unsigned long long)span) >> 32);
-        row = (int)(((long long)total - 1 - j) % cap);
-    } else {
-        row = have > 0 ? (int)(((unsigned long long)w.x * (unsigned long long)have) >> 32) : 0;
-    }
+    const int row = batch_row(b, B, have_host >= 0 ? have_host : *count, cap, seed, step, recent);
     if (lane == 0) t[b] = (ybuf[row] - stats[0]) / stats[1];
     for (int k = lane; k < K; k += 32)
         Xb[(size_t)b * K + k] = normalized(xbuf[(size_t)row * K + k], k, xmin, xmax);
@@ -728,16 +740,21 @@ rank_corr_kernel(const double *__restrict__ fk, const int *__restrict__ rows,
     }
 }
 
-// mean and standard deviation of the filled replay targets (one block)
-__global__ void stats_kernel(const float *__restrict__ ybuf, const int *count, int have_host, int cap,
-                             float *stats)
+// mean and standard deviation of the filled replay targets, on one cluster of
+// STATS_C CTAs (FP64 sums run at 1/64 of the FP32 rate: one CTA took 14 us for
+// 6144 targets), summed in a fixed order
+constexpr int STATS_C = 8;
+__global__ void __cluster_dims__(STATS_C, 1, 1) __launch_bounds__(512)
+stats_kernel(const float *__restrict__ ybuf, const int *count, int have_host, int cap, float *stats)
 {
-    __shared__ double s1[32], s2[32];
+    __shared__ double s1[16], s2[16], c1[STATS_C], c2[STATS_C];
+    cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
     const int n = min(have_host >= 0 ? have_host : *count, cap);
     double a = 0.0, b = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        a += ybuf[i];
-        b += (double)ybuf[i] * ybuf[i];
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += STATS_C * blockDim.x) {
+        const double y = ybuf[i];
+        a += y;
+        b += y * y;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -750,10 +767,20 @@ __global__ void stats_kernel(const float *__restrict__ ybuf, const int *count, i
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        double A = 0.0, Bs = 0.0;
+        a = b = 0.0;
         for (int w = 0; w < (int)blockDim.x / 32; ++w) {
-            A += s1[w];
-            Bs += s2[w];
+            a += s1[w];
+            b += s2[w];
+        }
+        *cluster.map_shared_rank(&c1[blockIdx.x], 0) = a;
+        *cluster.map_shared_rank(&c2[blockIdx.x], 0) = b;
+    }
+    cluster.sync();
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        double A = 0.0, Bs = 0.0;
+        for (int w = 0; w < STATS_C; ++w) {
+            A += c1[w];
+            Bs += c2[w];
         }
         double mu = n > 0 ? A / n : 0.0;
         double var = n > 1 ? Bs / n - mu * mu : 1.0;
@@ -888,6 +915,646 @@ __global__ void scatter_fill_kernel(const int *__restrict__ rows, const double *
     }
 }
 
+// ---------------------------------------------------------------------------
+// The whole network in one kernel per 128 batch rows (widths up to 256), for
+// which the layers' launches and the trips of Z and A through global memory
+// cost more than the products.  rows_kernel: a CTA gathers its rows, keeps both
+// weight matrices in shared memory and both accumulators in tensor memory
+// (columns 0 .. 255 for layer 1 and again for the data gradient, 256 .. 511 for
+// layer 2) and runs X W1 -> A1 W2 -> head; in training also dZ2 -> dZ2 W2 ->
+// dZ1 and the column sums of the bias and head gradients.  A thread owns one
+// row and every fourth group of 32 columns; its loops over them stay rolled
+// (each line runs once per launch, and unrolled the warps waited for
+// instructions).  Six training steps of 1024 pairs and a prediction of 1024, K =
+// 32, H = 256: 584 us layer by layer, 262 us here; bound by the latency of the
+// chain on 8 CTAs (29 us of a step's kernels under ncu, the gradients 15), with
+// the tensor core idle most of it.  grads_kernel: one CTA per 128 x 64
+// tile of a weight gradient, fed by bulk copies, with Adam on the tile.
+//
+// Layout of every matrix in shared memory and of the tiles in global memory
+// ("cores"): 8 x 8 BF16 blocks of 128 bytes (8 rows of 16 bytes), block (r / 8,
+// c / 8) at ((c / 8) RB + r / 8) 128 with RB the row blocks.  Read as a K-major
+// operand (k = c) its core strides are RB 128 along k and 128 along the rows; as
+// an MN-major operand (k = r) 128 along k and RB 128 along the columns: one copy
+// of W2 serves the forward and the data-gradient product, and a row range of the
+// batch tiles is what the weight gradients (k = batch) read, in whole
+// contiguous column blocks.
+// ---------------------------------------------------------------------------
+constexpr int ROWS_THREADS = 512, GRADS_THREADS = 256, HMAX = 256, BT = 128;   // BT: batch rows of a tile
+
+__host__ __device__ inline int up16(int n) { return (n + 15) / 16 * 16; }
+__host__ __device__ inline int up32(int n) { return (n + 31) / 32 * 32; }
+
+struct NetArgs {
+    int n, K, H;                           // batch rows, inputs, width
+    const __nv_bfloat16 *W1b, *W2b;
+    const float *b1, *b2, *w3, *b3;
+    const double *xmin, *xmax;
+    // rows: x[b] of a given batch, or drawn from the replay buffer (sample)
+    const float *x, *ybuf, *t;
+    int sample, step, recent, have_host, cap;
+    const int *count;
+    uint64_t seed;
+    const float *stats;
+    float *out;                            // predictions (no training), log misfit
+    // training: tiles [ceil(n / 128)] of X, A1, dZ2, dZ1, partial column sums
+    // [tiles][3][H] (w3, b2, b1), partial dy sum and loss
+    unsigned char *Xt, *A1t, *dZ2t, *dZ1t;
+    float *part, *part_dy;
+    double *part_loss;
+    int *err;
+};
+
+__device__ __forceinline__ int core_off(int r, int c, int RB)
+{
+    return ((c >> 3) * RB + (r >> 3)) * 128 + (r & 7) * 16 + (c & 7) * 2;
+}
+
+__device__ __forceinline__ void umma(unsigned d, unsigned long long ad, unsigned long long bd, unsigned idesc, bool acc)
+{
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
+                 " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+                 "l"(ad), "l"(bd), "r"(idesc), "r"((unsigned)acc)
+                 : "memory");
+}
+__device__ __forceinline__ void umma_commit(unsigned long long *bar)
+{
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(smem_u32(bar))
+                 : "memory");
+}
+
+// 32 columns of this thread's row from tensor memory
+__device__ __forceinline__ void tmem_row32(unsigned addr, float v[32])
+{
+    unsigned r[32];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,"
+        "%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(addr)
+        : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
+}
+
+// Sum over the warp's 32 rows (lanes) of 32 columns each lane holds: halves are
+// exchanged and added (16 + 8 + 4 + 2 + 1 shuffles); column `lane` ends in lane
+__device__ __forceinline__ float column_sum32(float v[32], int lane)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const bool hi = lane & o;
+#pragma unroll
+        for (int i = 0; i < o; ++i) {
+            const float keep = hi ? v[i + o] : v[i], send = hi ? v[i] : v[i + o];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+    return v[0];
+}
+
+// 8 consecutive values as BF16 into a core row (16 bytes)
+__device__ __forceinline__ void store8(unsigned char *dst, const float *v)
+{
+    __nv_bfloat162 h[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) h[q] = __floats2bfloat162_rn(v[2 * q], v[2 * q + 1]);
+    *reinterpret_cast<uint4 *>(dst) = *reinterpret_cast<uint4 *>(h);
+}
+
+// rows x cols (a multiple of 8) of a row-major BF16 matrix into cores at dst, by
+// asynchronous copies (the columns past `valid`, and odd widths, by plain stores)
+__device__ __forceinline__ void load_cores(unsigned char *dst, const __nv_bfloat16 *__restrict__ src, int rows,
+                                           int cols, int valid)
+{
+    const int nv = cols / 8, kg = nv % 4 == 0 ? 4 : 2, per = 8 * kg, bk = nv / kg, RB = rows / 8;
+    const bool vec = valid % 8 == 0 && ((size_t)src & 15) == 0;
+    for (int v = threadIdx.x; v < rows * nv; v += ROWS_THREADS) {
+        const int in = v % per, blk = v / per;
+        const int r = (blk / bk) * 8 + (in & 7), c = ((blk % bk) * kg + (in >> 3)) * 8;
+        unsigned char *d = dst + core_off(r, c, RB);
+        if (vec && c < valid) {
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_u32(d)), "l"(src + (size_t)r * valid + c)
+                         : "memory");
+        } else {
+            __nv_bfloat16 t[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) t[e] = c + e < valid ? src[(size_t)r * valid + c + e] : __float2bfloat16(0.f);
+            *reinterpret_cast<uint4 *>(d) = *reinterpret_cast<const uint4 *>(t);
+        }
+    }
+}
+
+// shared-memory plan of rows_kernel (bytes): W2, the A1 / dZ2 / dZ1 tile, then X
+// and W1 (whose place the column sums' partial sums take later) when they fit
+// beside, else X in the tile's place and W1 in W2's until layer 1 is done
+struct RowsPlan {
+    int w2, tile, x, w1, red, vec, bytes;
+    bool beside;
+};
+__host__ __device__ inline RowsPlan rows_plan(int K, int H)
+{
+    const int Kp = up16(K), xb = BT * Kp * 2, w1b = H * Kp * 2, redb = 3 * 4 * H * 4;
+    const int vecb = (3 * up32(H) + 2 * Kp + 2 * BT + HMAX / 32 * BT) * 4;
+    RowsPlan p{};
+    p.w2 = 0;
+    p.tile = H * H * 2;
+    const int end = p.tile + BT * H * 2, most = 227 * 1024 - 1024;
+    p.beside = end + xb + (w1b > redb ? w1b : redb) + vecb <= most;
+    if (p.beside) {
+        p.x = end;
+        p.w1 = p.red = end + xb;
+        p.vec = p.w1 + (w1b > redb ? w1b : redb);
+    } else {
+        // room for X and W1 where W2 and the tile will be
+        const int tile = p.tile > w1b ? p.tile : w1b;
+        p.tile = tile;
+        p.x = tile;
+        p.w1 = 0;
+        p.red = tile + (BT * H * 2 > xb ? BT * H * 2 : xb);
+        p.vec = p.red + redb;
+    }
+    p.bytes = p.vec + vecb;
+    return p;
+}
+
+template <bool TRAIN>
+__global__ void __launch_bounds__(ROWS_THREADS, 1) rows_kernel(const NetArgs a)
+{
+    extern __shared__ __align__(1024) unsigned char tsm[];
+    __shared__ __align__(8) unsigned long long mbar;
+    __shared__ unsigned tmem_base;
+    __shared__ int s_fail;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int K = a.K, H = a.H, Kp = up16(K), b0 = blockIdx.x * BT, tile = blockIdx.x;
+    const RowsPlan pl = rows_plan(K, H);
+    unsigned char *W2s = tsm + pl.w2, *T = tsm + pl.tile, *Xs = tsm + pl.x, *W1s = tsm + pl.w1;
+    float *red = reinterpret_cast<float *>(tsm + pl.red), *vec = reinterpret_cast<float *>(tsm + pl.vec);
+    const int Hp = up32(H);                 // the vectors are zero past H
+    float *b1 = vec, *b2 = vec + Hp, *w3 = vec + 2 * Hp, *lo = vec + 3 * Hp, *hi = lo + Kp, *ts = hi + Kp, *dys = ts + BT;
+    unsigned *on = reinterpret_cast<unsigned *>(dys + BT);       // signs of A1: [group of 32 columns][row]
+    if (tid == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&mbar)) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        s_fail = 0;
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&tmem_base)),
+                     "r"(512u)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    load_cores(W1s, a.W1b, H, Kp, K);
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+    if (pl.beside) load_cores(W2s, a.W2b, H, H, H);
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+    for (int h = tid; h < Hp; h += ROWS_THREADS) {
+        b1[h] = h < H ? a.b1[h] : 0.f;
+        b2[h] = h < H ? a.b2[h] : 0.f;
+        w3[h] = h < H ? a.w3[h] : 0.f;
+    }
+    for (int k = tid; k < K; k += ROWS_THREADS) {
+        lo[k] = (float)a.xmin[k];
+        hi[k] = (float)a.xmax[k];
+    }
+    __syncthreads();
+    // X: 16 rows per warp, scaled to [-1, 1]; zeros past the batch and the inputs
+    {
+        const int total = TRAIN && a.sample ? (a.have_host >= 0 ? a.have_host : *a.count) : 0;
+        constexpr int RW = BT / (ROWS_THREADS / 32);       // rows of a warp; lane i draws row i
+        const int bl = b0 + warp * RW + lane;
+        int row_l = bl;
+        float t_l = 0.f;
+        if (lane < RW && bl < a.n && TRAIN) {
+            if (a.sample) {
+                row_l = batch_row(bl, a.n, total, a.cap, a.seed, a.step, a.recent);
+                t_l = (a.ybuf[row_l] - a.stats[0]) / a.stats[1];
+            } else {
+                t_l = a.t[bl];
+            }
+        }
+        if (lane < RW) ts[warp * RW + lane] = t_l;
+#pragma unroll 4
+        for (int i = 0; i < RW; ++i) {
+            const int r = warp * RW + i, row = __shfl_sync(0xffffffffu, row_l, i);
+            for (int k = lane; k < Kp; k += 32) {
+                float v = 0.f;
+                if (b0 + r < a.n && k < K) v = 2.f * (a.x[(size_t)row * K + k] - lo[k]) / (hi[k] - lo[k]) - 1.f;
+                *reinterpret_cast<__nv_bfloat16 *>(Xs + core_off(r, k, BT / 8)) = __float2bfloat16(v);
+            }
+        }
+    }
+    asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    const unsigned tmem = tmem_base, idesc = umma_idesc(BT, H);
+    unsigned parity = 0;
+    // waits for the products issued last (bounded; gives up once)
+    auto products = [&] {
+        if (!mbar_wait_tc(smem_u32(&mbar), parity)) s_fail = 1;
+        parity ^= 1;
+        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    };
+    // a tile in shared memory to global memory (thread 0; its reads are awaited
+    // before the place is written again)
+    auto bulk_out = [&](unsigned char *dst, const unsigned char *src, unsigned bytes) {
+        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n" ::"l"(dst), "r"(smem_u32(src)),
+                     "r"(bytes)
+                     : "memory");
+        asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
+    };
+    auto bulk_read = [] { asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory"); };
+    if (tid == 0) {
+        for (int s = 0; s < Kp / 16; ++s)
+            umma(tmem, umma_desc(Xs + s * 2 * (BT / 8) * 128, BT / 8 * 128, 128),
+                 umma_desc(W1s + s * 2 * (H / 8) * 128, H / 8 * 128, 128), idesc, s > 0);
+        umma_commit(&mbar);
+        if (TRAIN) bulk_out(a.Xt + (size_t)tile * BT * Kp * 2, Xs, BT * Kp * 2);
+    }
+    products();
+    if (!pl.beside) {
+        if (TRAIN && tid == 0) bulk_read();        // X's place becomes the tile's
+        __syncthreads();
+        load_cores(W2s, a.W2b, H, H, H);
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+    // layer 1: A1 = relu(Z1 + b1) as the next product's operand; the signs are
+    // kept for the way back
+    const int r = 32 * (warp & 3) + lane, part = warp >> 2;
+    constexpr int STEP = 32 * (ROWS_THREADS / 128);      // columns from one group of a thread to its next
+    const bool real = b0 + r < a.n;
+    const unsigned trow = tmem + ((unsigned)(32 * (warp & 3)) << 16);
+#pragma unroll 1
+    for (int c0 = 32 * part; c0 < H; c0 += STEP) {
+        float v[32];
+        tmem_row32(trow + c0, v);
+        unsigned bits = 0u;
+#pragma unroll
+        for (int j = 0; j < 32; j += 4) {                // (columns past H go nowhere)
+            const float4 b = *reinterpret_cast<const float4 *>(b1 + c0 + j);
+            v[j] = fmaxf(v[j] + b.x, 0.f);
+            v[j + 1] = fmaxf(v[j + 1] + b.y, 0.f);
+            v[j + 2] = fmaxf(v[j + 2] + b.z, 0.f);
+            v[j + 3] = fmaxf(v[j + 3] + b.w, 0.f);
+        }
+        if (TRAIN) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) bits |= v[j] > 0.f ? 1u << j : 0u;
+        }
+        if (TRAIN) on[c0 / 32 * BT + r] = bits;
+#pragma unroll
+        for (int j = 0; j < 32; j += 8)
+            if (c0 + j < H) store8(T + core_off(r, c0 + j, BT / 8), v + j);
+    }
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    if (tid == 0) {
+        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+        for (int s = 0; s < H / 16; ++s)
+            umma(tmem + HMAX, umma_desc(T + s * 2 * (BT / 8) * 128, BT / 8 * 128, 128),
+                 umma_desc(W2s + s * 2 * (H / 8) * 128, H / 8 * 128, 128), idesc, s > 0);
+        umma_commit(&mbar);
+        if (TRAIN) bulk_out(a.A1t + (size_t)tile * BT * H * 2, T, BT * H * 2);
+    }
+    products();
+    // head: y = sum_h relu(Z2) w3 + b3 in the order of 32 strided partial sums
+    // added pairwise (one thread per row)
+    if (part == 0) {
+        float s[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j) s[j] = 0.f;
+#pragma unroll 1
+        for (int c0 = 0; c0 < H; c0 += 32) {
+            float v[32];
+            tmem_row32(trow + HMAX + c0, v);
+#pragma unroll
+            for (int j = 0; j < 32; j += 16) {           // (H is a multiple of 16)
+                if (c0 + j >= H) break;
+#pragma unroll
+                for (int i = j; i < j + 16; i += 4) {
+                    const float4 b = *reinterpret_cast<const float4 *>(b2 + c0 + i);
+                    const float4 w = *reinterpret_cast<const float4 *>(w3 + c0 + i);
+                    s[i] = fmaf(fmaxf(v[i] + b.x, 0.f), w.x, s[i]);
+                    s[i + 1] = fmaf(fmaxf(v[i + 1] + b.y, 0.f), w.y, s[i + 1]);
+                    s[i + 2] = fmaf(fmaxf(v[i + 2] + b.z, 0.f), w.z, s[i + 2]);
+                    s[i + 3] = fmaf(fmaxf(v[i + 3] + b.w, 0.f), w.w, s[i + 3]);
+                }
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int j = 0; j < o; ++j) s[j] += s[j + o];
+        const float y = s[0] + a.b3[0];
+        if (!TRAIN) {
+            if (real) a.out[b0 + r] = y * a.stats[1] + a.stats[0];
+        } else {
+            const float e = y - ts[r];
+            dys[r] = real ? e / (float)a.n : 0.f;
+            ts[r] = real ? e : 0.f;
+        }
+    }
+    if (TRAIN) {
+        if (tid == 0) bulk_read();                 // A1 has left the tile
+        __syncthreads();
+        if (warp == ROWS_THREADS / 32 - 1) {       // the tile's dy sum and loss (fixed order)
+            float sd = 0.f;
+            double sl = 0.0;
+            for (int i = lane; i < BT; i += 32) {
+                sd += dys[i];
+                sl += (double)ts[i] * ts[i];
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                sd += __shfl_down_sync(0xffffffffu, sd, o);
+                sl += __shfl_down_sync(0xffffffffu, sl, o);
+            }
+            if (lane == 0) {
+                a.part_dy[tile] = sd;
+                a.part_loss[tile] = sl;
+            }
+        }
+        // dZ2 = dy w3 [Z2 > 0]; column sums of relu(Z2) dy and of dZ2
+        const float dy = dys[r];
+#pragma unroll 1
+        for (int c0 = 32 * part; c0 < H; c0 += STEP) {
+            float v[32], z[32];
+            tmem_row32(trow + HMAX + c0, z);
+#pragma unroll
+            for (int j = 0; j < 32; j += 4) {            // (columns past H go nowhere)
+                const float4 b = *reinterpret_cast<const float4 *>(b2 + c0 + j);
+                const float4 w = *reinterpret_cast<const float4 *>(w3 + c0 + j);
+                auto one = [&](int i, float bb, float ww) {
+                    const float zz = z[i] + bb;
+                    v[i] = zz > 0.f && real ? dy * ww : 0.f;
+                    z[i] = real ? fmaxf(zz, 0.f) * dy : 0.f;
+                };
+                one(j, b.x, w.x);
+                one(j + 1, b.y, w.y);
+                one(j + 2, b.z, w.z);
+                one(j + 3, b.w, w.w);
+            }
+#pragma unroll
+            for (int j = 0; j < 32; j += 8)
+                if (c0 + j < H) store8(T + core_off(r, c0 + j, BT / 8), v + j);
+            const float sw = column_sum32(z, lane), sb = column_sum32(v, lane);
+            if (c0 + lane < H) {
+                red[(0 * 4 + (warp & 3)) * H + c0 + lane] = sw;
+                red[(1 * 4 + (warp & 3)) * H + c0 + lane] = sb;
+            }
+        }
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+        __syncthreads();
+        if (tid == 0) {
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            // dA1 = dZ2 W2: W2 read MN-major (k = its rows)
+            for (int s = 0; s < H / 16; ++s)
+                umma(tmem, umma_desc(T + s * 2 * (BT / 8) * 128, BT / 8 * 128, 128),
+                     umma_desc(W2s + s * 2 * 128, 128, H / 8 * 128), idesc | (1u << 16), s > 0);
+            umma_commit(&mbar);
+            bulk_out(a.dZ2t + (size_t)tile * BT * H * 2, T, BT * H * 2);
+        }
+        products();
+        if (tid == 0) bulk_read();                 // dZ2 has left the tile
+        __syncthreads();
+#pragma unroll 1
+        for (int c0 = 32 * part; c0 < H; c0 += STEP) {
+            float v[32];
+            tmem_row32(trow + c0, v);
+            const unsigned bits = real ? on[c0 / 32 * BT + r] : 0u;
+#pragma unroll
+            for (int j = 0; j < 32; ++j) v[j] = (bits >> j & 1u) ? v[j] : 0.f;
+#pragma unroll
+            for (int j = 0; j < 32; j += 8)
+                if (c0 + j < H) store8(T + core_off(r, c0 + j, BT / 8), v + j);
+            const float sb = column_sum32(v, lane);
+            if (c0 + lane < H) red[(2 * 4 + (warp & 3)) * H + c0 + lane] = sb;
+        }
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+        __syncthreads();
+        if (tid == 0) bulk_out(a.dZ1t + (size_t)tile * BT * H * 2, T, BT * H * 2);
+        for (int e = tid; e < 3 * H; e += ROWS_THREADS) {
+            const int q = e / H, h = e % H;
+            a.part[((size_t)tile * 3 + q) * H + h] =
+                ((red[(q * 4) * H + h] + red[(q * 4 + 1) * H + h]) + red[(q * 4 + 2) * H + h]) + red[(q * 4 + 3) * H + h];
+        }
+    }
+    if (tid == 0) {
+        asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory");   // every tile is written
+        if (s_fail) atomicExch(a.err, EMPSO_TIMEOUT);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(512u) : "memory");
+}
+
+// Weight gradients of `tiles` batch tiles: the CTAs of g_W2 (128 x 64 tiles of
+// dZ2^T A1), of g_W1 (dZ1^T X), and one for the vectors.  The batch tiles come
+// in by bulk copies, GSTAGES in flight (a tile's columns are contiguous
+// blocks); the accumulator takes them in batch order.  With `adam` the
+// gradient's tile is applied at once, else it is written.
+constexpr int GT_N = 64, GSTAGES = 4, GA_BYTES = 128 * BT * 2, GB_BYTES = GT_N * BT * 2;
+constexpr int GRADS_SMEM = GSTAGES * (GA_BYTES + GB_BYTES);
+
+struct GradArgs {
+    int n, tiles, K, H, adam;
+    const unsigned char *Xt, *A1t, *dZ2t, *dZ1t;
+    const float *part, *part_dy;
+    const double *part_loss;
+    float *p, *g, *m, *v, *loss;
+    long long off_b1, off_W2, off_b2, off_w3, off_b3;
+    __nv_bfloat16 *W1b, *W2b;
+    AdamStep step;
+    int *err;
+};
+
+__device__ __forceinline__ void apply_grad(const GradArgs &a, long long e, float gi, __nv_bfloat16 *wb)
+{
+    if (!a.adam) {
+        a.g[e] = gi;
+        return;
+    }
+    float m = a.m[e], v = a.v[e];
+    const float w = a.step(a.p[e], gi, m, v);
+    a.m[e] = m;
+    a.v[e] = v;
+    a.p[e] = w;
+    if (wb) *wb = __float2bfloat16(w);
+}
+
+__host__ __device__ inline int grad_tiles(int H, int N) { return (H + 127) / 128 * ((N + GT_N - 1) / GT_N); }
+
+__global__ void __launch_bounds__(GRADS_THREADS, 1) grads_kernel(const GradArgs a)
+{
+    extern __shared__ __align__(1024) unsigned char tsm[];
+    __shared__ __align__(8) unsigned long long full[GSTAGES], done[GSTAGES];
+    __shared__ unsigned tmem_base;
+    __shared__ int s_fail;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, H = a.H, Kp = up16(a.K);
+    const int n2 = grad_tiles(H, H), n1 = grad_tiles(H, Kp);
+    int b = blockIdx.x;
+    if (b >= n2 + n1) {
+        // w3, b2, b1: the batch tiles' partial sums in order; b3 and the loss
+        for (int e = tid; e < 3 * H; e += GRADS_THREADS) {
+            const int q = e / H, h = e % H;
+            float s = 0.f;
+#pragma unroll 8
+            for (int t = 0; t < a.tiles; ++t) s += a.part[((size_t)t * 3 + q) * H + h];
+            apply_grad(a, (q == 0 ? a.off_w3 : (q == 1 ? a.off_b2 : a.off_b1)) + h, s, nullptr);
+        }
+        if (tid == 0) {
+            float s = 0.f;
+            double l = 0.0;
+            for (int t = 0; t < a.tiles; ++t) {
+                s += a.part_dy[t];
+                l += a.part_loss[t];
+            }
+            apply_grad(a, a.off_b3, s, nullptr);
+            if (a.loss) *a.loss = (float)(0.5 * l / a.n);
+        }
+        return;
+    }
+    const bool second = b < n2;
+    if (!second) b -= n2;
+    const int N = second ? H : Kp, Nv = second ? H : a.K;          // columns staged, columns that exist
+    const int nx = (N + GT_N - 1) / GT_N, m0 = b / nx * 128, n0 = b % nx * GT_N;
+    const int mc = min(128, H - m0), nc = min(GT_N, N - n0);
+    const unsigned char *At = second ? a.dZ2t : a.dZ1t, *Bt = second ? a.A1t : a.Xt;
+    const size_t a_tile = (size_t)BT * H * 2, b_tile = (size_t)BT * N * 2;
+    const size_t a_ofs = (size_t)(m0 / 8) * (BT / 8) * 128, b_ofs = (size_t)(n0 / 8) * (BT / 8) * 128;
+    const unsigned a_bytes = mc * BT * 2, b_bytes = nc * BT * 2;
+    if (tid == 0) {
+        for (int i = 0; i < GSTAGES; ++i) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&full[i])) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&done[i])) : "memory");
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        s_fail = 0;
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&tmem_base)),
+                     "r"(64u)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    const unsigned tmem = tmem_base;
+    if (tid == 0) {
+        const unsigned idesc = umma_idesc(128, nc) | (1u << 15) | (1u << 16);     // both MN-major (k = batch row)
+        auto fetch = [&](int t) {
+            const int st = t % GSTAGES;
+            unsigned char *As = tsm + st * (GA_BYTES + GB_BYTES), *Bs = As + GA_BYTES;
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(&full[st])),
+                         "r"(a_bytes + b_bytes)
+                         : "memory");
+            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
+                             smem_u32(As)),
+                         "l"(At + t * a_tile + a_ofs), "r"(a_bytes), "r"(smem_u32(&full[st]))
+                         : "memory");
+            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
+                             smem_u32(Bs)),
+                         "l"(Bt + t * b_tile + b_ofs), "r"(b_bytes), "r"(smem_u32(&full[st]))
+                         : "memory");
+        };
+        for (int t = 0; t < min(a.tiles, GSTAGES); ++t) fetch(t);
+        for (int t = 0; t < a.tiles; ++t) {
+            const int st = t % GSTAGES;
+            unsigned char *As = tsm + st * (GA_BYTES + GB_BYTES), *Bs = As + GA_BYTES;
+            if (!mbar_wait_tc(smem_u32(&full[st]), (t / GSTAGES) & 1)) s_fail = 1;
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            for (int s = 0; s < BT / 16; ++s)
+                umma(tmem, umma_desc(As + s * 2 * 128, 128, BT / 8 * 128), umma_desc(Bs + s * 2 * 128, 128, BT / 8 * 128),
+                     idesc, t > 0 || s > 0);
+            umma_commit(&done[st]);
+            // the stage of the tile before this one takes the tile after next
+            const int f = t - 1 + GSTAGES;
+            if (t >= 1 && f < a.tiles) {
+                if (!mbar_wait_tc(smem_u32(&done[(t - 1) % GSTAGES]), ((t - 1) / GSTAGES) & 1)) s_fail = 1;
+                fetch(f);
+            }
+        }
+        const int t = a.tiles - 1;                 // the last commit covers every product before it
+        if (!mbar_wait_tc(smem_u32(&done[t % GSTAGES]), (t / GSTAGES) & 1)) s_fail = 1;
+    }
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    // the tile through shared memory, so that parameters are read and written in rows
+    constexpr int GP = GT_N + 4;
+    float *G = reinterpret_cast<float *>(tsm);
+    for (int c0 = 32 * (warp >> 2); c0 < GT_N; c0 += 64) {
+        float v[32];
+        tmem_row32(tmem + ((unsigned)(32 * (warp & 3)) << 16) + c0, v);
+#pragma unroll
+        for (int j = 0; j < 32; j += 4)
+            *reinterpret_cast<float4 *>(G + (32 * (warp & 3) + lane) * GP + c0 + j) =
+                make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+    }
+    __syncthreads();
+    const long long off = second ? a.off_W2 : 0;
+    __nv_bfloat16 *Wb = second ? a.W2b : a.W1b;
+    if (!s_fail && a.adam && Nv % 4 == 0 && off % 4 == 0) {
+        // four parameters at a time, the loads of four such groups together
+        constexpr int Q = GT_N / 4, IT = 128 * Q / GRADS_THREADS, UN = 4;
+        for (int i0 = 0; i0 < IT; i0 += UN) {
+            float4 p[UN], m[UN], v[UN];
+            long long q[UN];
+            bool on[UN];
+#pragma unroll
+            for (int i = 0; i < UN; ++i) {
+                const int e = tid + (i0 + i) * GRADS_THREADS, r = e / Q, c = e % Q * 4;
+                on[i] = r < mc && n0 + c < Nv && c < nc;
+                q[i] = (long long)(m0 + r) * Nv + n0 + c;
+                if (on[i]) {
+                    p[i] = *reinterpret_cast<const float4 *>(a.p + off + q[i]);
+                    m[i] = *reinterpret_cast<const float4 *>(a.m + off + q[i]);
+                    v[i] = *reinterpret_cast<const float4 *>(a.v + off + q[i]);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < UN; ++i) {
+                if (!on[i]) continue;
+                const int e = tid + (i0 + i) * GRADS_THREADS, r = e / Q, c = e % Q * 4;
+                const float4 gi = *reinterpret_cast<const float4 *>(G + r * GP + c);
+                p[i].x = a.step(p[i].x, gi.x, m[i].x, v[i].x);
+                p[i].y = a.step(p[i].y, gi.y, m[i].y, v[i].y);
+                p[i].z = a.step(p[i].z, gi.z, m[i].z, v[i].z);
+                p[i].w = a.step(p[i].w, gi.w, m[i].w, v[i].w);
+                *reinterpret_cast<float4 *>(a.p + off + q[i]) = p[i];
+                *reinterpret_cast<float4 *>(a.m + off + q[i]) = m[i];
+                *reinterpret_cast<float4 *>(a.v + off + q[i]) = v[i];
+                const __nv_bfloat162 h0 = __floats2bfloat162_rn(p[i].x, p[i].y), h1 = __floats2bfloat162_rn(p[i].z, p[i].w);
+                reinterpret_cast<__nv_bfloat162 *>(Wb + q[i])[0] = h0;
+                reinterpret_cast<__nv_bfloat162 *>(Wb + q[i])[1] = h1;
+            }
+        }
+    } else if (!s_fail) {
+        for (int e = tid; e < 128 * GT_N; e += GRADS_THREADS) {
+            const int r = e / GT_N, c = e % GT_N;
+            if (r >= mc || n0 + c >= Nv || c >= nc) continue;
+            const long long q = (long long)(m0 + r) * Nv + n0 + c;
+            apply_grad(a, off + q, G[r * GP + c], Wb + q);
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(64u) : "memory");
+    if (tid == 0 && s_fail) atomicExch(a.err, EMPSO_TIMEOUT);
+}
+
 inline int blocks_for(long long n, int per = 256)
 {
     long long b = (n + per - 1) / per;
@@ -900,11 +1567,29 @@ inline int blocks_for(long long n, int per = 256)
 // host-side launchers used by api.cu
 // ---------------------------------------------------------------------------
 
-// opt the tcgen05 products into their two chunk buffers (current device)
-cudaError_t sur_prepare_tc()
+// opt the tcgen05 kernels into their shared memory (current device)
+cudaError_t sur_prepare_tc(const SurDev &)
 {
-    return cudaFuncSetAttribute(jobs_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
+    cudaError_t e = cudaFuncSetAttribute(jobs_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(grads_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, GRADS_SMEM);
+    // (the largest plan: the attribute is the kernel's, not the network's)
+    constexpr int MOST = 227 * 1024 - 1024;
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(rows_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, MOST);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(rows_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, MOST);
+    return e;
 }
+
+// does the whole-network kernel take this network (and backend)?
+bool sur_whole(const SurDev &s)
+{
+    return s.tc && s.err && s.H <= HMAX && up16(s.K) <= HMAX && rows_plan(s.K, s.H).bytes <= 227 * 1024 - 1024;
+}
+
+// bytes of one batch tile's X, A1, dZ2 and dZ1 and its partial sums
+size_t sur_tile_bytes(int K, int H) { return (size_t)BT * (up16(K) + 3 * H) * 2 + 12 * (size_t)H + 16; }
 
 namespace {
 
@@ -919,8 +1604,100 @@ cudaError_t hidden_layers(const SurDev &s, const __nv_bfloat16 *Xb, int n, cudaS
 
 }  // namespace
 
-// gradient of the half-MSE on batch (Xb [n][K] BF16, t [n]) into s.g; loss
+namespace {
+
+AdamStep adam_step(SurDev &s)
+{
+    s.t += 1;
+    return {s.lr, s.beta1, s.beta2, s.eps, 1.f - powf(s.beta1, (float)s.t), 1.f - powf(s.beta2, (float)s.t)};
+}
+
+NetArgs net_args(const SurDev &s, int n)
+{
+    NetArgs a{};
+    a.n = n;
+    a.K = s.K;
+    a.H = s.H;
+    a.W1b = s.W1b;
+    a.W2b = s.W2b;
+    a.b1 = s.p + s.off_b1;
+    a.b2 = s.p + s.off_b2;
+    a.w3 = s.p + s.off_w3;
+    a.b3 = s.p + s.off_b3;
+    a.xmin = s.xmin;
+    a.xmax = s.xmax;
+    a.stats = s.stats;
+    a.err = s.err;
+    return a;
+}
+
+// forward, backward and (step given) the update, two launches; the rows of `a`
+// are set.  The tiles lie one kind after the other in s.tiles.
+cudaError_t whole_step(const SurDev &s, NetArgs a, const AdamStep *step, float *loss, cudaStream_t st)
+{
+    const int T = (a.n + BT - 1) / BT, Kp = up16(s.K);
+    unsigned char *q = s.tiles;
+    auto take = [&](size_t bytes) {
+        unsigned char *p = q;
+        q += bytes * T;
+        return p;
+    };
+    a.Xt = take((size_t)BT * Kp * 2);
+    a.A1t = take((size_t)BT * s.H * 2);
+    a.dZ2t = take((size_t)BT * s.H * 2);
+    a.dZ1t = take((size_t)BT * s.H * 2);
+    a.part_loss = reinterpret_cast<double *>(take(8));
+    a.part = reinterpret_cast<float *>(take(12 * (size_t)s.H));
+    a.part_dy = reinterpret_cast<float *>(take(4));
+    rows_kernel<true><<<T, ROWS_THREADS, rows_plan(s.K, s.H).bytes, st>>>(a);
+    GradArgs g{};
+    g.n = a.n;
+    g.tiles = T;
+    g.K = s.K;
+    g.H = s.H;
+    g.adam = step != nullptr;
+    if (step) g.step = *step;
+    g.Xt = a.Xt;
+    g.A1t = a.A1t;
+    g.dZ2t = a.dZ2t;
+    g.dZ1t = a.dZ1t;
+    g.part = a.part;
+    g.part_dy = a.part_dy;
+    g.part_loss = a.part_loss;
+    g.p = s.p;
+    g.g = s.g;
+    g.m = s.m;
+    g.v = s.v;
+    g.loss = loss;
+    g.off_b1 = s.off_b1;
+    g.off_W2 = s.off_W2;
+    g.off_b2 = s.off_b2;
+    g.off_w3 = s.off_w3;
+    g.off_b3 = s.off_b3;
+    g.W1b = s.W1b;
+    g.W2b = s.W2b;
+    g.err = s.err;
+    grads_kernel<<<grad_tiles(s.H, s.H) + grad_tiles(s.H, Kp) + 1, GRADS_THREADS, GRADS_SMEM, st>>>(g);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+// gradient of the half-MSE on batch (x [n][K] positions, t [n]) into s.g; loss
 // to *loss (device float, may be null)
+cudaError_t sur_gradient(const SurDev &s, const float *x, const float *t, int n, float *loss, cudaStream_t st)
+{
+    if (sur_whole(s)) {
+        NetArgs a = net_args(s, n);
+        a.x = x;
+        a.t = t;
+        return whole_step(s, a, nullptr, loss, st);
+    }
+    cudaError_t e = sur_normalize(s, x, n, s.Xb, st);
+    return e ? e : sur_backward(s, s.Xb, t, n, loss, st);
+}
+
+// the same from BF16 rows, layer by layer
 cudaError_t sur_backward(const SurDev &s, const __nv_bfloat16 *Xb, const float *t, int n,
                          float *loss, cudaStream_t st)
 {
@@ -956,10 +1733,7 @@ cudaError_t sur_backward(const SurDev &s, const __nv_bfloat16 *Xb, const float *
 
 cudaError_t sur_adam(SurDev &s, cudaStream_t st)
 {
-    s.t += 1;
-    const float c1 = 1.f - powf(s.beta1, (float)s.t), c2 = 1.f - powf(s.beta2, (float)s.t);
-    adam_kernel<<<blocks_for(s.n_params), 256, 0, st>>>(s.p, s.g, s.m, s.v, s.n_params, s.lr, s.beta1,
-                                                        s.beta2, s.eps, c1, c2, s.W1b,
+    adam_kernel<<<blocks_for(s.n_params), 256, 0, st>>>(s.p, s.g, s.m, s.v, s.n_params, adam_step(s), s.W1b,
                                                         (long long)s.H * s.K, s.W2b, s.off_W2,
                                                         (long long)s.H * s.H);
     return cudaGetLastError();
@@ -982,6 +1756,13 @@ cudaError_t sur_normalize(const SurDev &s, const float *x, int n, __nv_bfloat16 
 
 cudaError_t sur_predict(const SurDev &s, const float *x, int n, float *logphi, cudaStream_t st)
 {
+    if (sur_whole(s)) {
+        NetArgs a = net_args(s, n);
+        a.x = x;
+        a.out = logphi;
+        rows_kernel<false><<<(n + BT - 1) / BT, ROWS_THREADS, rows_plan(s.K, s.H).bytes, st>>>(a);
+        return cudaGetLastError();
+    }
     cudaError_t e;
     if ((e = sur_normalize(s, x, n, s.Xb, st))) return e;
     if ((e = hidden_layers(s, s.Xb, n, st))) return e;
@@ -1000,8 +1781,23 @@ cudaError_t sur_append(const SurDev &s, const float *x, const double *misfit, co
 cudaError_t sur_train(SurDev &s, int steps, int B, cudaStream_t st, int have)
 {
     cudaError_t e;
-    stats_kernel<<<1, 1024, 0, st>>>(s.ybuf, s.count, have, s.cap, s.stats);
+    stats_kernel<<<STATS_C, 512, 0, st>>>(s.ybuf, s.count, have, s.cap, s.stats);
     for (int i = 0; i < steps; ++i) {
+        if (sur_whole(s)) {
+            NetArgs a = net_args(s, B);
+            a.sample = 1;
+            a.x = s.xbuf;
+            a.ybuf = s.ybuf;
+            a.count = s.count;
+            a.have_host = have;
+            a.cap = s.cap;
+            a.seed = s.seed;
+            a.step = s.sample_step++;
+            a.recent = s.recent;
+            const AdamStep step = adam_step(s);
+            if ((e = whole_step(s, a, &step, s.loss, st))) return e;
+            continue;
+        }
         batch_kernel<<<(B * 32 + 255) / 256, 256, 0, st>>>(B, s.K, s.count, have, s.cap, s.seed, s.sample_step++,
                                                            s.recent, s.xbuf, s.ybuf, s.stats, s.xmin, s.xmax, s.tb,
                                                            s.Xb);
