@@ -24,7 +24,9 @@
 // Laplacian), and leaves its traces for adj_residual_kernel;
 // at order 16 on the plain streaming kernel; adj_fwd_kernel is the per-step
 // form for grids none of them can hold, which keeps its time levels in two
-// adjoint slots and writes the same history.  The per-step kernels here run over all instances at once
+// adjoint slots and writes the same history.  The backward pass is one launch
+// for all steps on groups of co-resident CTAs (adj_group_kernel) where that is
+// faster (adj_group_split).  The per-step kernels run over all instances at once
 // (blockIdx.y = instance), one launch per time step (the time loops replay as
 // one CUDA graph).  They stage the fields their Laplacians read in
 // shared-memory tiles and give each thread a few rows of one float4 group.
@@ -35,6 +37,7 @@
 
 #include "internal.cuh"
 #include "stencil.cuh"
+#include "wave_group.cuh"
 
 namespace empso {
 
@@ -523,6 +526,321 @@ __global__ void __launch_bounds__(T2_THREADS, 4) adj_step2_kernel(GridDev g, con
     }
 }
 
+// ---------------------------------------------------------------------------
+// The whole backward pass of an instance on a group of co-resident CTAs
+// (wave_group.cuh): one launch for all steps.  A thread keeps its run of rows
+// through the pass, so mu^{k+1}, mu^{k+2} and G of its points stay in shared
+// memory ([row][thread], no other thread reads them), and only Q^k = f a mu^k,
+// which the neighbours' Laplacians need, goes through global memory (two slots
+// in turn), beside the streams of f a and of the history: 17 B a point-step and
+// no launch where the per-step kernels move 30 B and re-stage their tiles'
+// halos.  One more CTA of the group scatters the receiver term of the step
+// after.  Every point's operations are those of adj_step_kernel in the same
+// order.
+// ---------------------------------------------------------------------------
+template <int R>
+__device__ __forceinline__ void sweep_adjoint(const GridDev &g, const AdjInst &in, const float4 *cur, float4 *nxt,
+                                              const float4 *hist, float4 *jf, int p4, int q, int j0, int len, bool act,
+                                              int lmax, float4 *xb, float4 *mu1, float4 *mu2, float4 *gs, float c0,
+                                              const float *cx, const float *cz, const SrcCorner &sc, float rn)
+{
+    constexpr int N = Window<R>::N, XG = XRow<R>::XG, ZERO = XRow<R>::ZERO, LEN = XRow<R>::LEN, O = 4 * XG;
+    const int lane = threadIdx.x & 31, NQ = g.NQ;
+    const unsigned pb = (unsigned)p4 * 16u;
+    unsigned o_st = ((unsigned)(j0 + HALO) * (unsigned)p4 + HALO4 + q) * 16u;
+    unsigned o_pf = o_st + PF * pb, o_w = o_st + (R + PF) * pb, o_ez = (unsigned)(j0 + HALO + PF) * 4u;
+    const char *cu = reinterpret_cast<const char *>(cur), *hu = reinterpret_cast<const char *>(hist);
+    const char *bu = reinterpret_cast<const char *>(in.B), *zu = reinterpret_cast<const char *>(g.ez);
+    char *ju = reinterpret_cast<char *>(jf), *nu = reinterpret_cast<char *>(nxt);
+    auto ld = [](const char *p, unsigned o) { return *reinterpret_cast<const float4 *>(p + o); };
+    auto ldg = [](const char *p, unsigned o) { return __ldg(reinterpret_cast<const float4 *>(p + o)); };
+    auto lds = [](const char *p, unsigned o) { return __ldcs(reinterpret_cast<const float4 *>(p + o)); };
+    const bool left = lane < XG, edge = left || lane >= 32 - XG;
+    const int src = left ? 0 : 31;
+    const int qe = __shfl_sync(0xffffffffu, q, src), je = __shfl_sync(0xffffffffu, j0, src);
+    unsigned o_e =
+        ((unsigned)(je + HALO) * (unsigned)p4 + HALO4 + qe + (left ? lane - XG : lane - (32 - XG) + 1)) * 16u;
+    float4 *eslot = xb + (left ? lane : lane + 2 * XG), *own = xb + XG + lane;
+    const float4 *x_l = xb + (q >= 1 ? XG + lane - 1 : ZERO), *x_r = xb + (q + 1 < NQ ? XG + lane + 1 : ZERO);
+    const float4 *x_l2 = xb + (q >= 2 ? XG + lane - 2 : ZERO), *x_r2 = xb + (q + 2 < NQ ? XG + lane + 2 : ZERO);
+    const float4 ex = __ldg(reinterpret_cast<const float4 *>(g.ex + HALO) + q);
+    const bool xpad = __any_sync(0xffffffffu, ex.x != 0.f || ex.y != 0.f || ex.z != 0.f || ex.w != 0.f);
+    const int ks = sc.I0 >= 4 * q - 1 && sc.I0 <= 4 * q + 3 ? sc.J0 - j0 : -2;
+    const bool ragged = 4 * q + 3 >= g.NX;             // lanes past the last column stay zero
+    const int jr0 = in.jr0 - j0, jr1 = in.jr1 - j0;    // run rows that may hold a receiver term
+    const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 w[N], lu[U], bv[U], jv[U];
+    float ez[U];
+#pragma unroll
+    for (int m = 0; m < 2 * R + PF; ++m)
+        if (m - 2 * R < lmax) w[m] = ld(cu, o_st + (m - R) * pb);
+#pragma unroll
+    for (int m = 0; m < PF; ++m) {
+        if (m < lmax) {
+            lu[m] = lds(hu, o_st + m * pb);
+            bv[m] = ldg(bu, o_st + m * pb);
+            jv[m] = m >= jr0 && m <= jr1 ? ld(ju, o_st + m * pb) : zero4;
+            ez[m] = __ldg(g.ez + j0 + HALO + m);
+            if (edge) cp_async16(eslot + m * LEN, cu + o_e + m * pb);
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    }
+    o_e += PF * pb;
+    auto row = [&](const int k0, const int kk, const bool full) {
+        const int k = k0 + kk, s = kk * LEN, kn = (kk + PF) % U;
+        const float4 *wl = w + kk;
+        own[s] = wl[R];
+        asm volatile("cp.async.wait_group %0;\n" ::"n"(PF - 1) : "memory");
+        __syncwarp();
+        if (full || k + PF < lmax) {
+            w[kk + 2 * R + PF] = ld(cu, o_w);
+            lu[kn] = lds(hu, o_pf);
+            // the next step's history into L2 (it comes from HBM)
+            asm volatile("prefetch.global.L2 [%0];\n" ::"l"(hu - 4 * g.field + o_pf));
+            bv[kn] = ldg(bu, o_pf);
+            jv[kn] = k + PF >= jr0 && k + PF <= jr1 ? ld(ju, o_pf) : zero4;
+            ez[kn] = __ldg(reinterpret_cast<const float *>(zu + o_ez));
+            if (edge) cp_async16(eslot + kn * LEN, cu + o_e);
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+        float xs[4 * (2 * XG + 1)];
+        if (XG == 1) xline1(x_l[s], wl[R], x_r[s], xs);
+        else xline2(x_l2[s], x_l[s], wl[R], x_r[s], x_r2[s], xs);
+        // the Laplacian summed as written (lap4_tile_sum's order, packed)
+        float2 o01 = __fmul2_rn(splat2(c0), f2(xs[O], xs[O + 1])), o23 = __fmul2_rn(splat2(c0), f2(xs[O + 2], xs[O + 3]));
+#pragma unroll
+        for (int m = 1; m <= R; ++m) {
+            const float2 z01 = __fadd2_rn(lo2(wl[R - m]), lo2(wl[R + m])), z23 = __fadd2_rn(hi2(wl[R - m]), hi2(wl[R + m]));
+            const float2 s01 = (m & 1) ? f2(xs[O - m] + xs[O + m], xs[O + 1 - m] + xs[O + 1 + m])
+                                       : __fadd2_rn(f2(xs[O - m], xs[O + 1 - m]), f2(xs[O + m], xs[O + 1 + m]));
+            const float2 s23 = (m & 1) ? f2(xs[O + 2 - m] + xs[O + 2 + m], xs[O + 3 - m] + xs[O + 3 + m])
+                                       : __fadd2_rn(f2(xs[O + 2 - m], xs[O + 3 - m]), f2(xs[O + 2 + m], xs[O + 3 + m]));
+            o01 = __ffma2_rn(splat2(cz[m]), z01, __ffma2_rn(splat2(cx[m]), s01, o01));
+            o23 = __ffma2_rn(splat2(cz[m]), z23, __ffma2_rn(splat2(cx[m]), s23, o23));
+        }
+        const int e = k * WAVE_THREADS;
+        float4 a1 = zero4, a2 = zero4, gg = zero4;
+        if (full || k < len) {
+            a1 = mu1[e];
+            a2 = mu2[e];
+            gg = gs[e];
+        }
+        const float2 j01 = lo2(jv[kk]), j23 = hi2(jv[kk]);
+        float2 l01 = lo2(lu[kk]), l23 = hi2(lu[kk]);
+        if (k == ks || k == ks + 1) {                   // the source term of the forward step
+            const int J = j0 + k, I = 4 * q;
+            l01 = f2(fmaf(src_weight(sc, I, J), rn, l01.x), fmaf(src_weight(sc, I + 1, J), rn, l01.y));
+            l23 = f2(fmaf(src_weight(sc, I + 2, J), rn, l23.x), fmaf(src_weight(sc, I + 3, J), rn, l23.y));
+        }
+        // mu^k = 2 f mu^{k+1} + L Q - (1 - t) f mu^{k+2} + J, G += mu^k f (L u + s)
+        float2 m01, m23, g01, g23;
+        const float2 one = splat2(1.f), mone = splat2(-1.f), two = splat2(2.f);
+        if (ez[kk] != 0.f || xpad) {
+            const float2 z = splat2(ez[kk]);
+            const float2 t01 = __fadd2_rn(lo2(ex), z), t23 = __fadd2_rn(hi2(ex), z);
+            const float2 d01 = __fadd2_rn(one, t01), d23 = __fadd2_rn(one, t23);
+            const float2 f01 = quot2(one, d01), f23 = quot2(one, d23);
+            const float2 h01 = __fmul2_rn(__fadd2_rn(t01, mone), f01), h23 = __fmul2_rn(__fadd2_rn(t23, mone), f23);
+            m01 = __fadd2_rn(__ffma2_rn(h01, lo2(a2), __ffma2_rn(__fmul2_rn(two, f01), lo2(a1), o01)), j01);
+            m23 = __fadd2_rn(__ffma2_rn(h23, hi2(a2), __ffma2_rn(__fmul2_rn(two, f23), hi2(a1), o23)), j23);
+            if (ragged) {
+                const int I = 4 * q;
+                m01 = f2(I < g.NX ? m01.x : 0.f, I + 1 < g.NX ? m01.y : 0.f);
+                m23 = f2(I + 2 < g.NX ? m23.x : 0.f, I + 3 < g.NX ? m23.y : 0.f);
+            }
+            g01 = __ffma2_rn(quot2(m01, d01), l01, lo2(gg));
+            g23 = __ffma2_rn(quot2(m23, d23), l23, hi2(gg));
+        } else {
+            m01 = __fadd2_rn(__ffma2_rn(mone, lo2(a2), __ffma2_rn(two, lo2(a1), o01)), j01);
+            m23 = __fadd2_rn(__ffma2_rn(mone, hi2(a2), __ffma2_rn(two, hi2(a1), o23)), j23);
+            if (ragged) {
+                const int I = 4 * q;
+                m01 = f2(I < g.NX ? m01.x : 0.f, I + 1 < g.NX ? m01.y : 0.f);
+                m23 = f2(I + 2 < g.NX ? m23.x : 0.f, I + 3 < g.NX ? m23.y : 0.f);
+            }
+            g01 = __ffma2_rn(m01, l01, lo2(gg));
+            g23 = __ffma2_rn(m23, l23, hi2(gg));
+        }
+        if (act && (full || k < len)) {
+            mu2[e] = make_float4(m01.x, m01.y, m23.x, m23.y);
+            gs[e] = make_float4(g01.x, g01.y, g23.x, g23.y);
+            float2 q01 = __fmul2_rn(lo2(bv[kk]), m01), q23 = __fmul2_rn(hi2(bv[kk]), m23);
+            if (ragged) {
+                const int I = 4 * q;
+                q01 = f2(I < g.NX ? q01.x : 0.f, I + 1 < g.NX ? q01.y : 0.f);
+                q23 = f2(I + 2 < g.NX ? q23.x : 0.f, I + 3 < g.NX ? q23.y : 0.f);
+            }
+            *reinterpret_cast<float4 *>(nu + o_st) = make_float4(q01.x, q01.y, q23.x, q23.y);
+            if (j01.x != 0.f || j01.y != 0.f || j23.x != 0.f || j23.y != 0.f) *reinterpret_cast<float4 *>(ju + o_st) = zero4;
+        }
+        o_st += pb;
+        o_pf += pb;
+        o_w += pb;
+        o_e += pb;
+        o_ez += 4u;
+    };
+    int k0 = 0;
+    for (; k0 + U - 1 + PF < lmax; k0 += U) {
+#pragma unroll
+        for (int kk = 0; kk < U; ++kk) row(k0, kk, true);
+#pragma unroll
+        for (int m = 0; m < N - U; ++m) w[m] = w[m + U];
+    }
+    for (; k0 < lmax; k0 += U) {
+#pragma unroll
+        for (int kk = 0; kk < U; ++kk)
+            if (k0 + kk < lmax) row(k0, kk, false);
+#pragma unroll
+        for (int m = 0; m < N - U; ++m) w[m] = w[m + U];
+    }
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+}
+
+constexpr int ADJ_CTAS = 2;                                  // per SM
+
+// scatter_receiver_term for a CTA that does it every step: corners and weights
+// are kept, the next step's residuals are requested while this one's are
+// scattered (loaded in the step that scatters them, in each of the four passes,
+// they made the step: 8 us)
+constexpr int SCATTER_PER = 8;                               // receivers of a thread
+struct Scatter {
+    long long at[SCATTER_PER];                               // offset of the first corner
+    float w[SCATTER_PER][4], e[SCATTER_PER];
+    bool fits;
+
+    __device__ __forceinline__ void request(const AdjInst &in, int kk)
+    {
+#pragma unroll
+        for (int i = 0; i < SCATTER_PER; ++i) {
+            const int r = threadIdx.x + i * WAVE_THREADS;
+            e[i] = r < in.nrec && kk >= 1 ? in.E[(long long)(kk - 1) * in.nrec + r] : 0.f;
+        }
+    }
+    __device__ __forceinline__ void begin(const GridDev &g, const AdjInst &in)
+    {
+        fits = in.nrec <= SCATTER_PER * WAVE_THREADS;
+        if (!fits) return;
+#pragma unroll
+        for (int i = 0; i < SCATTER_PER; ++i) {
+            const int r = threadIdx.x + i * WAVE_THREADS;
+            const float2 p = r < in.nrec ? in.rec[r] : make_float2(0.f, 0.f);
+            const SrcCorner c = src_corner(p.x, p.y, g);
+            at[i] = (long long)(c.J0 + HALO) * g.pitch + c.I0 + HALO;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) w[i][q] = in.w * c.w[q];
+        }
+        request(in, g.nt);
+    }
+    __device__ __forceinline__ void step(const GridDev &g, const AdjInst &in, int kk)
+    {
+        if (!fits) {
+            scatter_receiver_term(g, in, kk);
+            return;
+        }
+        float v[SCATTER_PER];
+#pragma unroll
+        for (int i = 0; i < SCATTER_PER; ++i) v[i] = e[i];
+        request(in, kk - 1);
+        float *J = in.J + (long long)(kk % 4) * g.field;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+#pragma unroll
+            for (int i = 0; i < SCATTER_PER; ++i)
+                if (threadIdx.x + i * WAVE_THREADS < in.nrec)
+                    atomicAdd(J + at[i] + (q >> 1) * g.pitch + (q & 1), w[i][q] * v[i]);
+            __syncthreads();
+        }
+    }
+};
+
+// Group `blockIdx.x / (group + 1)` takes instances gid, gid + groups, ...; its
+// CTAs 0 .. group - 1 sweep, the last one scatters.  rows: the rows of shared
+// memory a thread has (at least its run's).
+template <int R>
+__global__ void __launch_bounds__(WAVE_THREADS, ADJ_CTAS)
+adj_group_kernel(GridDev gk, const AdjInst *__restrict__ insts, int n_inst, int group, int rows, int *ws, int *err)
+{
+    extern __shared__ float4 tsm4[];
+    __shared__ float4 xrows[WAVE_THREADS / 32 * U * XRow<R>::LEN];
+    __shared__ GridDev g;
+    __shared__ int s_fail;
+    const int n = group + 1, gid = blockIdx.x / n, rank = blockIdx.x % n, groups = gridDim.x / n;
+    const int tid = threadIdx.x, lane = tid & 31, nth = group * WAVE_THREADS;
+    unsigned *count = reinterpret_cast<unsigned *>(ws + WS_LINE * (1 + gid));
+    unsigned target = 0;
+    float4 *xb = xrows + (tid >> 5) * U * XRow<R>::LEN;
+    if (lane < U) xb[lane * XRow<R>::LEN + XRow<R>::ZERO] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (tid == 0) {
+        s_fail = 0;
+        g = gk;
+    }
+    __syncthreads();
+    float4 *mA = tsm4 + tid, *mB = mA + rows * WAVE_THREADS, *gs = mB + rows * WAVE_THREADS;
+    const int NQ = g.NQ, p4 = g.pitch / 4;
+    const int nseg = max(1, min(g.NZ, nth / NQ)), items = NQ * nseg;
+    const int i0 = rank * WAVE_THREADS + tid - lane, item = min(i0 + lane, items - 1);
+    const bool sweeper = rank < group && i0 < items, act = sweeper && i0 + lane < items;
+    const int q = item % NQ, seg = item / NQ;
+    const int j0 = (int)((long long)seg * g.NZ / nseg), j1 = (int)((long long)(seg + 1) * g.NZ / nseg), len = j1 - j0;
+    const int lmax = __reduce_max_sync(0xffffffffu, len);
+    float cx[R + 1], cz[R + 1];
+#pragma unroll
+    for (int m = 0; m <= R; ++m) {
+        cx[m] = g.cxm[m];
+        cz[m] = g.czm[m];
+    }
+    bool ok = true;
+    if (rank == group) {
+        for (int i = gid; i < n_inst && ok; i += groups) {
+            const AdjInst in = insts[i];
+            Scatter scatter;
+            scatter.begin(g, in);
+            for (int k = g.nt; k >= 0 && ok; --k) {      // J^k while step k + 1 is swept
+                if (k >= 1) scatter.step(g, in, k);
+                ok = group_barrier(count, target, n, &s_fail);
+            }
+        }
+    } else {
+        for (int i = gid; i < n_inst && ok; i += groups) {
+            const AdjInst in = insts[i];
+            const SrcCorner sc = src_corner(in.sx, in.sz, g);
+            for (int k = 0; k < rows; ++k) {
+                const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+                mA[k * WAVE_THREADS] = z;
+                mB[k * WAVE_THREADS] = z;
+                gs[k * WAVE_THREADS] = z;
+            }
+            ok = group_barrier(count, target, n, &s_fail);
+            for (int k = g.nt; k >= 1 && ok; --k) {
+                // mu^{k+1} and mu^{k+2} of this thread (mu^k takes the latter's place)
+                const bool even = ((g.nt - k) & 1) == 0;
+                if (sweeper)
+                    sweep_adjoint<R>(g, in, reinterpret_cast<const float4 *>(in.mu + (long long)((k + 1) % 2) * g.field),
+                                     reinterpret_cast<float4 *>(in.mu + (long long)(k % 2) * g.field),
+                                     reinterpret_cast<const float4 *>(in.H + (long long)k * g.field),
+                                     reinterpret_cast<float4 *>(in.J + (long long)(k % 4) * g.field), p4, q, j0, len, act,
+                                     lmax, xb, even ? mA : mB, even ? mB : mA, gs, cx[0], cx, cz, sc,
+                                     g.wavelet[k - 1] / (g.hx * g.hz));
+                ok = group_barrier(count, target, n, &s_fail);
+            }
+            if (ok && act) {
+                float4 *G4 = reinterpret_cast<float4 *>(in.G) + (size_t)(j0 + HALO) * p4 + HALO4 + q;
+                for (int k = 0; k < len; ++k) G4[(size_t)k * p4] = gs[k * WAVE_THREADS];
+            }
+        }
+    }
+    if (tid == 0 && s_fail) atomicExch(err, EMPSO_TIMEOUT);
+}
+
+using AdjGroupFn = void (*)(GridDev, const AdjInst *, int, int, int, int *, int *);
+AdjGroupFn adj_group_fn(int R)
+{
+    if (R == 8) return adj_group_kernel<8>;
+    if (R == 4) return adj_group_kernel<4>;
+    return R == 2 ? adj_group_kernel<2> : adj_group_kernel<1>;
+}
+size_t adj_group_smem(int rows) { return sizeof(float4) * 3 * (size_t)rows * WAVE_THREADS; }
+
 // residual e_n = R u^{n+1} - d_obs,n (one block per instance), u^{n+1} in the
 // rotating slots of the per-step forward pass
 __global__ void adj_record_kernel(GridDev g, const AdjInst *__restrict__ insts, int n)
@@ -705,6 +1023,73 @@ cudaError_t launch_adj_residual(const GridDev &g, const AdjInst *insts, int n_in
     const long long n = (long long)g.nt * rec_max;
     adj_residual_kernel<<<dim3((unsigned)std::min<long long>((n + 255) / 256, 64), n_inst), 256, 0, st>>>(insts, g.nt);
     return cudaGetLastError();
+}
+
+// Instances in flight and sweeping CTAs each (one more scatters) of the
+// persistent backward pass: the least estimated time among the splits whose
+// threads' rows fit shared memory; group 0 when none does, or when up to radius
+// 4 it would take more than one round of instances (the per-step kernels read
+// less there, two steps a launch or more blocks in flight).  Whole gradients on
+// the 461 x 151 grid, order 8, per-step and persistent backward pass: 4 shots
+// 13.2 and 11.2 ms, 8 shots 16.2 and 13.5, 16 shots 24.5 and 23.6, 32 shots (two
+// rounds) 42.4 and 44.2; order 16, 4 shots of the 921 x 301 grid: 84.5 and 56.0.
+AdjSplit adj_group_split(const GridDev &g, long long n_inst, size_t smem_optin)
+{
+    constexpr int RUN_EXTRA = 10;
+    AdjSplit best{};
+    int sms = 0, dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return best;
+    const int per = ADJ_CTAS, ctas = std::min(sms * per, WAVE_MAX_CTAS);
+    // an SM's shared memory, less each CTA's static part and the system's 1 KB
+    const size_t room = smem_optin / per - (12u << 10);
+    double cost = 0.0;
+    for (long long f = 1; f <= std::min<long long>(n_inst, ctas / 2); ++f) {
+        const int n = (int)(ctas / f) - 1, nseg = std::min(g.NZ, n * WAVE_THREADS / g.NQ);
+        if (nseg < 1) break;                     // one run of rows per thread
+        const int rows = (g.NZ + nseg - 1) / nseg;
+        if (adj_group_smem(rows) > room || (g.R <= 4 && f < n_inst)) continue;
+        const double c = (double)((n_inst + f - 1) / f) * (rows + RUN_EXTRA);
+        if (best.group == 0 || c < cost) {
+            cost = c;
+            best.flight = (int)f;
+            best.group = std::min(n, (g.NQ * nseg + WAVE_THREADS - 1) / WAVE_THREADS);
+            best.rows = rows;
+        }
+    }
+    // (the CTAs of a group wait for one another: all must be resident)
+    int fit = 0;
+    if (best.group &&
+        (cudaFuncSetAttribute(adj_group_fn(g.R), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)adj_group_smem(best.rows)) != cudaSuccess ||
+         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, adj_group_fn(g.R), WAVE_THREADS, adj_group_smem(best.rows)) !=
+             cudaSuccess ||
+         fit < per)) {
+        cudaGetLastError();
+        best = AdjSplit{};
+    }
+    return best;
+}
+
+cudaError_t launch_adj_group(const GridDev &g, const AdjInst *insts, int n_inst, const AdjSplit &s, void *ws, int *err,
+                             cudaStream_t st)
+{
+    const AdjGroupFn fn = adj_group_fn(g.R);
+    const size_t smem = adj_group_smem(s.rows);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ws, 0, sizeof(int) * WS_LINE * (1 + (size_t)s.flight), st);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.gridDim = dim3(s.flight * (s.group + 1), 1, 1);
+    cfg.blockDim = dim3(WAVE_THREADS, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, fn, g, insts, n_inst, s.group, s.rows, (int *)ws, err);
 }
 
 cudaError_t launch_adj_backward(const GridDev &g, const AdjInst *insts, int n_inst, int n_all, int rec_threads,

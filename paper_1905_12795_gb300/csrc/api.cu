@@ -1299,21 +1299,17 @@ empso_status gradient_impl(empso_ctx *ctx, const float *vel, int M, const empso_
     // step.  Its cluster size: a gradient has few instances (shots x models),
     // so the rounds of clusters matter, not only the SMs busy: the fewest
     // rounds x rows per CTA (a round's time follows the rows a CTA sweeps),
-    // then the most SMs busy, over C <= 12 when some such size fits (13..16
-    // measured slower at every shot count: 16 shots on the 461 x 151 grid
-    // took 28.5 ms at C = 12, 30.2 at the 15 clusters of C = 9, 31.3-32.4 at
-    // C = 13..16).
+    // then the most SMs busy.  Whole gradients on the 461 x 151 grid: 1, 4 and 8
+    // shots at C = 12 9.35, 11.27 and 13.40 ms, at C = 16 8.96, 10.88 and 16.92
+    // (two rounds); 16 shots 23.27 at C = 12, 24.75 at C = 9, 26.4 at C = 16.
     int rC = 0, r_threads = 0, r_nc = 0, r_rows = 0;
     size_t r_smem = 0;
-    // (the cluster kernels hold stencils up to radius 4: order 16 takes the
-    // per-step launches)
+    // (the cluster kernels hold stencils up to radius 4)
     const bool want_res = g.R <= MAX_R_FAST &&
                           (ctx->kernel_kind == EMPSO_KERNEL_AUTO || ctx->kernel_kind == EMPSO_KERNEL_RESIDENT);
     if (want_res) {
         long long best_cost = 0, best_sms = 0;
-        // C <= 12 first; 13 .. 16 only for grids that need them
-        for (int pass = 0; pass < 2 && !rC; ++pass)
-        for (int C = pass == 0 ? 1 : 13; C <= (pass == 0 ? 12 : 16); ++C)
+        for (int C = 1; C <= 16; ++C)
             for (const int rows : resident_runs(ctx->forced_rows)) {
                 if (ctx->forced_C > 0 && C != ctx->forced_C) continue;
                 if (!resident_fits(g, C, rec_max, ctx->smem_optin, rows)) continue;
@@ -1349,10 +1345,11 @@ empso_status gradient_impl(empso_ctx *ctx, const float *vel, int M, const empso_
     if (g.R > MAX_R_FAST) split = wave_split(&gp, 1, g.R, I, by_l2, true);
     if ((l2 || g.R > MAX_R_FAST) && split.group < 1)
         return fail(ctx, EMPSO_CUDA_ERROR, "gradient: occupancy of the forward kernel");
-    if (split.group) {
+    const AdjSplit back = adj_group_split(g, I, ctx->smem_optin);
+    if (split.group || back.group) {
         if ((rc = adj_grow(ctx, &W.wave_ws, &W.wave_ws_cap, wave_ws_bytes(), nullptr))) return rc;
-        if ((rc = adj_grow(ctx, &W.slots, &W.slots_cap, F / 2 * split.flight, nullptr))) return rc;
     }
+    if (split.group && (rc = adj_grow(ctx, &W.slots, &W.slots_cap, F / 2 * split.flight, nullptr))) return rc;
     const size_t r_ofs = ((size_t)I * sizeof(Inst) + 255) / 256 * 256;
     const bool table = rC || split.group;
     if (table) {
@@ -1446,7 +1443,9 @@ empso_status gradient_impl(empso_ctx *ctx, const float *vel, int M, const empso_
             if (ce == cudaSuccess && !forward_only)
                 ce = cudaMemsetAsync(W.mu, 0, sizeof(float) * F * 4 * I, ctx->cap_stream);
         }
-        if (ce == cudaSuccess && !forward_only) {
+        if (ce == cudaSuccess && !forward_only && back.group) {
+            ce = launch_adj_group(g, W.insts, (int)I, back, W.wave_ws, ctx->dev_err, ctx->cap_stream);
+        } else if (ce == cudaSuccess && !forward_only) {
             // instances [c I / n, (c + 1) I / n) on chain c (chain 0 on the
             // capture stream), forked after the forward pass and joined at the end
             const int want = ctx->grad_chains > 0 ? ctx->grad_chains : (I >= 16 ? 4 : 1);

@@ -127,6 +127,14 @@ cudaError_t launch_adj_residual(const GridDev &g, const AdjInst *insts, int n_in
 // n + 1
 cudaError_t launch_adj_backward(const GridDev &g, const AdjInst *insts, int n_inst, int n_all, int rec_threads,
                                 cudaStream_t st);
+// the backward pass as one launch on groups of co-resident CTAs (ws:
+// wave_ws_bytes(); every instance's mu, J zero before)
+struct AdjSplit {
+    int flight, group, rows;
+};
+AdjSplit adj_group_split(const GridDev &g, long long n_inst, size_t smem_optin);
+cudaError_t launch_adj_group(const GridDev &g, const AdjInst *insts, int n_inst, const AdjSplit &s, void *ws, int *err,
+                             cudaStream_t st);
 // T: scratch of max(M * NZ * nx floats, M * S * 64 doubles), 8-byte aligned
 // (the misfit partials, then the x-folded gradient)
 cudaError_t launch_adj_finish(const GridDev &g, const AdjInst *insts, int M, int S, const float *vel,
