@@ -428,9 +428,8 @@ __device__ __forceinline__ void colsum_cols(const ColSum &c, int bx)
         if (h < c.H)
 #pragma unroll 8
             for (int b = ty; b < c.n; b += CS_T) {
-                float v = c.X[(size_t)b * c.H + h];
-                if (c.wrow) v = fmaxf(v, 0.f) * c.wrow[b];
-                s += v;
+                const float v = c.X[(size_t)b * c.H + h];
+                s = c.wrow ? fmaf(fmaxf(v, 0.f), c.wrow[b], s) : s + v;
             }
         red[ty][tx] = s;
     }
@@ -615,13 +614,15 @@ __global__ void head_kernel(const float *__restrict__ Z2, int n, int H, const fl
     }
 }
 
-// Adam on FP32 master weights
+// Adam on FP32 master weights.  The contractions are written out: left to the
+// compiler, each kernel's differ in the last bit, and where a gradient is near
+// zero the moments' ratio carries that bit into an update of the order of lr.
 struct AdamStep {
     float lr, b1, b2, eps, c1, c2;
     __device__ __forceinline__ float operator()(float w, float gi, float &m, float &v) const
     {
-        m = b1 * m + (1.f - b1) * gi;
-        v = b2 * v + (1.f - b2) * gi * gi;
+        m = fmaf(1.f - b1, gi, b1 * m);
+        v = fmaf((1.f - b2) * gi, gi, b2 * v);
         return w - lr * (m / c1) / (sqrtf(v / c2) + eps);
     }
 };
@@ -922,11 +923,14 @@ __global__ void scatter_fill_kernel(const int *__restrict__ rows, const double *
 // weight matrices in shared memory and both accumulators in tensor memory
 // (columns 0 .. 255 for layer 1 and again for the data gradient, 256 .. 511 for
 // layer 2) and runs X W1 -> A1 W2 -> head; in training also dZ2 -> dZ2 W2 ->
-// dZ1 and the column sums of the bias and head gradients.  A thread owns one
+// dZ1, and writes relu(Z2), dZ2 and dZ1 in FP32 for the column sums of the bias
+// and head gradients, which grads_kernel takes over the whole batch in the
+// layer-by-layer path's order: partial sums per tile (262 us) differ from it in the last
+// bit, and Adam turns that into 1e-3 where a gradient is near zero.  A thread owns one
 // row and every fourth group of 32 columns; its loops over them stay rolled
 // (each line runs once per launch, and unrolled the warps waited for
 // instructions).  Six training steps of 1024 pairs and a prediction of 1024, K =
-// 32, H = 256: 584 us layer by layer, 262 us here; bound by the latency of the
+// 32, H = 256: 584 us layer by layer, 281 us here; bound by the latency of the
 // chain on 8 CTAs (29 us of a step's kernels under ncu, the gradients 15), with
 // the tensor core idle most of it.  grads_kernel: one CTA per 128 x 64
 // tile of a weight gradient, fed by bulk copies, with Adam on the tile.
@@ -957,10 +961,10 @@ struct NetArgs {
     uint64_t seed;
     const float *stats;
     float *out;                            // predictions (no training), log misfit
-    // training: tiles [ceil(n / 128)] of X, A1, dZ2, dZ1, partial column sums
-    // [tiles][3][H] (w3, b2, b1), partial dy sum and loss
+    // training: tiles [ceil(n / 128)] of X, A1, dZ2, dZ1 in BF16; relu(Z2), dZ2,
+    // dZ1 in FP32 [tiles][3][H][128]; dy [tiles][128]; the tiles' losses
     unsigned char *Xt, *A1t, *dZ2t, *dZ1t;
-    float *part, *part_dy;
+    float *cols, *dy;
     double *part_loss;
     int *err;
 };
@@ -1001,22 +1005,6 @@ __device__ __forceinline__ void tmem_row32(unsigned addr, float v[32])
     for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
 }
 
-// Sum over the warp's 32 rows (lanes) of 32 columns each lane holds: halves are
-// exchanged and added (16 + 8 + 4 + 2 + 1 shuffles); column `lane` ends in lane
-__device__ __forceinline__ float column_sum32(float v[32], int lane)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const bool hi = lane & o;
-#pragma unroll
-        for (int i = 0; i < o; ++i) {
-            const float keep = hi ? v[i + o] : v[i], send = hi ? v[i] : v[i + o];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-        }
-    }
-    return v[0];
-}
-
 // 8 consecutive values as BF16 into a core row (16 bytes)
 __device__ __forceinline__ void store8(unsigned char *dst, const float *v)
 {
@@ -1050,33 +1038,32 @@ __device__ __forceinline__ void load_cores(unsigned char *dst, const __nv_bfloat
 }
 
 // shared-memory plan of rows_kernel (bytes): W2, the A1 / dZ2 / dZ1 tile, then X
-// and W1 (whose place the column sums' partial sums take later) when they fit
+// and W1 when they fit
 // beside, else X in the tile's place and W1 in W2's until layer 1 is done
 struct RowsPlan {
-    int w2, tile, x, w1, red, vec, bytes;
+    int w2, tile, x, w1, vec, bytes;
     bool beside;
 };
 __host__ __device__ inline RowsPlan rows_plan(int K, int H)
 {
-    const int Kp = up16(K), xb = BT * Kp * 2, w1b = H * Kp * 2, redb = 3 * 4 * H * 4;
+    const int Kp = up16(K), xb = BT * Kp * 2, w1b = H * Kp * 2;
     const int vecb = (3 * up32(H) + 2 * Kp + 2 * BT + HMAX / 32 * BT) * 4;
     RowsPlan p{};
     p.w2 = 0;
     p.tile = H * H * 2;
     const int end = p.tile + BT * H * 2, most = 227 * 1024 - 1024;
-    p.beside = end + xb + (w1b > redb ? w1b : redb) + vecb <= most;
+    p.beside = end + xb + w1b + vecb <= most;
     if (p.beside) {
         p.x = end;
-        p.w1 = p.red = end + xb;
-        p.vec = p.w1 + (w1b > redb ? w1b : redb);
+        p.w1 = end + xb;
+        p.vec = p.w1 + w1b;
     } else {
         // room for X and W1 where W2 and the tile will be
         const int tile = p.tile > w1b ? p.tile : w1b;
         p.tile = tile;
         p.x = tile;
         p.w1 = 0;
-        p.red = tile + (BT * H * 2 > xb ? BT * H * 2 : xb);
-        p.vec = p.red + redb;
+        p.vec = tile + (BT * H * 2 > xb ? BT * H * 2 : xb);
     }
     p.bytes = p.vec + vecb;
     return p;
@@ -1093,7 +1080,7 @@ __global__ void __launch_bounds__(ROWS_THREADS, 1) rows_kernel(const NetArgs a)
     const int K = a.K, H = a.H, Kp = up16(K), b0 = blockIdx.x * BT, tile = blockIdx.x;
     const RowsPlan pl = rows_plan(K, H);
     unsigned char *W2s = tsm + pl.w2, *T = tsm + pl.tile, *Xs = tsm + pl.x, *W1s = tsm + pl.w1;
-    float *red = reinterpret_cast<float *>(tsm + pl.red), *vec = reinterpret_cast<float *>(tsm + pl.vec);
+    float *vec = reinterpret_cast<float *>(tsm + pl.vec);
     const int Hp = up32(H);                 // the vectors are zero past H
     float *b1 = vec, *b2 = vec + Hp, *w3 = vec + 2 * Hp, *lo = vec + 3 * Hp, *hi = lo + Kp, *ts = hi + Kp, *dys = ts + BT;
     unsigned *on = reinterpret_cast<unsigned *>(dys + BT);       // signs of A1: [group of 32 columns][row]
@@ -1265,24 +1252,26 @@ __global__ void __launch_bounds__(ROWS_THREADS, 1) rows_kernel(const NetArgs a)
     if (TRAIN) {
         if (tid == 0) bulk_read();                 // A1 has left the tile
         __syncthreads();
-        if (warp == ROWS_THREADS / 32 - 1) {       // the tile's dy sum and loss (fixed order)
-            float sd = 0.f;
+        if (warp == ROWS_THREADS / 32 - 1) {       // the tile's loss (fixed order)
             double sl = 0.0;
-            for (int i = lane; i < BT; i += 32) {
-                sd += dys[i];
-                sl += (double)ts[i] * ts[i];
-            }
+            for (int i = lane; i < BT; i += 32) sl += (double)ts[i] * ts[i];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                sd += __shfl_down_sync(0xffffffffu, sd, o);
-                sl += __shfl_down_sync(0xffffffffu, sl, o);
-            }
-            if (lane == 0) {
-                a.part_dy[tile] = sd;
-                a.part_loss[tile] = sl;
-            }
+            for (int o = 16; o > 0; o >>= 1) sl += __shfl_down_sync(0xffffffffu, sl, o);
+            if (lane == 0) a.part_loss[tile] = sl;
         }
-        // dZ2 = dy w3 [Z2 > 0]; column sums of relu(Z2) dy and of dZ2
+        if (part == 0) a.dy[(size_t)tile * BT + r] = dys[r];
+        // what grads_kernel sums over the batch: relu(Z2), dZ2, dZ1 in FP32, a column's
+        // rows side by side
+        float *const col = a.cols + (size_t)tile * 3 * H * BT + r;
+        auto keep = [&](int q, int c0, const float v[32]) {
+#pragma unroll
+            for (int j = 0; j < 32; j += 16) {           // (H is a multiple of 16)
+                if (c0 + j >= H) break;
+#pragma unroll
+                for (int i = j; i < j + 16; ++i) col[(size_t)(q * H + c0 + i) * BT] = v[i];
+            }
+        };
+        // dZ2 = dy w3 [Z2 > 0]
         const float dy = dys[r];
 #pragma unroll 1
         for (int c0 = 32 * part; c0 < H; c0 += STEP) {
@@ -1295,7 +1284,7 @@ __global__ void __launch_bounds__(ROWS_THREADS, 1) rows_kernel(const NetArgs a)
                 auto one = [&](int i, float bb, float ww) {
                     const float zz = z[i] + bb;
                     v[i] = zz > 0.f && real ? dy * ww : 0.f;
-                    z[i] = real ? fmaxf(zz, 0.f) * dy : 0.f;
+                    z[i] = real ? fmaxf(zz, 0.f) : 0.f;
                 };
                 one(j, b.x, w.x);
                 one(j + 1, b.y, w.y);
@@ -1305,11 +1294,8 @@ __global__ void __launch_bounds__(ROWS_THREADS, 1) rows_kernel(const NetArgs a)
 #pragma unroll
             for (int j = 0; j < 32; j += 8)
                 if (c0 + j < H) store8(T + core_off(r, c0 + j, BT / 8), v + j);
-            const float sw = column_sum32(z, lane), sb = column_sum32(v, lane);
-            if (c0 + lane < H) {
-                red[(0 * 4 + (warp & 3)) * H + c0 + lane] = sw;
-                red[(1 * 4 + (warp & 3)) * H + c0 + lane] = sb;
-            }
+            keep(0, c0, z);
+            keep(1, c0, v);
         }
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
@@ -1336,18 +1322,12 @@ __global__ void __launch_bounds__(ROWS_THREADS, 1) rows_kernel(const NetArgs a)
 #pragma unroll
             for (int j = 0; j < 32; j += 8)
                 if (c0 + j < H) store8(T + core_off(r, c0 + j, BT / 8), v + j);
-            const float sb = column_sum32(v, lane);
-            if (c0 + lane < H) red[(2 * 4 + (warp & 3)) * H + c0 + lane] = sb;
+            keep(2, c0, v);
         }
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
         __syncthreads();
         if (tid == 0) bulk_out(a.dZ1t + (size_t)tile * BT * H * 2, T, BT * H * 2);
-        for (int e = tid; e < 3 * H; e += ROWS_THREADS) {
-            const int q = e / H, h = e % H;
-            a.part[((size_t)tile * 3 + q) * H + h] =
-                ((red[(q * 4) * H + h] + red[(q * 4 + 1) * H + h]) + red[(q * 4 + 2) * H + h]) + red[(q * 4 + 3) * H + h];
-        }
     }
     if (tid == 0) {
         asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory");   // every tile is written
@@ -1360,7 +1340,7 @@ __global__ void __launch_bounds__(ROWS_THREADS, 1) rows_kernel(const NetArgs a)
 }
 
 // Weight gradients of `tiles` batch tiles: the CTAs of g_W2 (128 x 64 tiles of
-// dZ2^T A1), of g_W1 (dZ1^T X), and one for the vectors.  The batch tiles come
+// dZ2^T A1), of g_W1 (dZ1^T X), and those of the vectors.  The batch tiles come
 // in by bulk copies, GSTAGES in flight (a tile's columns are contiguous
 // blocks); the accumulator takes them in batch order.  With `adam` the
 // gradient's tile is applied at once, else it is written.
@@ -1370,7 +1350,7 @@ constexpr int GRADS_SMEM = GSTAGES * (GA_BYTES + GB_BYTES);
 struct GradArgs {
     int n, tiles, K, H, adam;
     const unsigned char *Xt, *A1t, *dZ2t, *dZ1t;
-    const float *part, *part_dy;
+    const float *cols, *dy;
     const double *part_loss;
     float *p, *g, *m, *v, *loss;
     long long off_b1, off_W2, off_b2, off_w3, off_b3;
@@ -1393,6 +1373,8 @@ __device__ __forceinline__ void apply_grad(const GradArgs &a, long long e, float
     if (wb) *wb = __float2bfloat16(w);
 }
 
+constexpr int SUM_COLS = 4;              // columns of a warp of the vectors' CTAs
+__host__ __device__ inline int vector_ctas(int H) { return 1 + (3 * H + GRADS_THREADS / 32 * SUM_COLS - 1) / (GRADS_THREADS / 32 * SUM_COLS); }
 __host__ __device__ inline int grad_tiles(int H, int N) { return (H + 127) / 128 * ((N + GT_N - 1) / GT_N); }
 
 __global__ void __launch_bounds__(GRADS_THREADS, 1) grads_kernel(const GradArgs a)
@@ -1405,24 +1387,48 @@ __global__ void __launch_bounds__(GRADS_THREADS, 1) grads_kernel(const GradArgs 
     const int n2 = grad_tiles(H, H), n1 = grad_tiles(H, Kp);
     int b = blockIdx.x;
     if (b >= n2 + n1) {
-        // w3, b2, b1: the batch tiles' partial sums in order; b3 and the loss
-        for (int e = tid; e < 3 * H; e += GRADS_THREADS) {
-            const int q = e / H, h = e % H;
+        b -= n2 + n1;
+        if (b == 0) {                                    // b3 and the loss
             float s = 0.f;
-#pragma unroll 8
-            for (int t = 0; t < a.tiles; ++t) s += a.part[((size_t)t * 3 + q) * H + h];
-            apply_grad(a, (q == 0 ? a.off_w3 : (q == 1 ? a.off_b2 : a.off_b1)) + h, s, nullptr);
-        }
-        if (tid == 0) {
-            float s = 0.f;
-            double l = 0.0;
-            for (int t = 0; t < a.tiles; ++t) {
-                s += a.part_dy[t];
-                l += a.part_loss[t];
+            sum_all(a.dy, a.n, &s);
+            if (tid == 0) {
+                apply_grad(a, a.off_b3, s, nullptr);
+                double l = 0.0;
+                for (int t = 0; t < a.tiles; ++t) l += a.part_loss[t];
+                if (a.loss) *a.loss = (float)(0.5 * l / a.n);
             }
-            apply_grad(a, a.off_b3, s, nullptr);
-            if (a.loss) *a.loss = (float)(0.5 * l / a.n);
+            return;
         }
+        // w3, b2, b1: a warp per SUM_COLS columns; lane i adds rows i, i + 32, ..,
+        // then the lanes' sums are added pairwise (the order of the layer-by-layer path)
+        const int e0 = ((b - 1) * (GRADS_THREADS / 32) + warp) * SUM_COLS;
+        float s[SUM_COLS];
+        const float *src[SUM_COLS];
+#pragma unroll
+        for (int i = 0; i < SUM_COLS; ++i) {
+            s[i] = 0.f;
+            src[i] = a.cols + (size_t)min(e0 + i, 3 * H - 1) * BT + lane;
+        }
+        for (int t = 0; t < a.tiles; ++t)
+#pragma unroll
+            for (int k = 0; k < BT; k += 32) {
+                const float dy = a.dy[t * BT + k + lane];
+#pragma unroll
+                for (int i = 0; i < SUM_COLS; ++i) {
+                    const float v = src[i][(size_t)t * 3 * H * BT + k];
+                    s[i] = e0 + i < H ? fmaf(v, dy, s[i]) : s[i] + v;
+                }
+            }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int i = 0; i < SUM_COLS; ++i) s[i] += __shfl_down_sync(0xffffffffu, s[i], o);
+        if (lane == 0)
+#pragma unroll
+            for (int i = 0; i < SUM_COLS; ++i) {
+                const int e = e0 + i, q = e / H, h = e % H;
+                if (e < 3 * H) apply_grad(a, (q == 0 ? a.off_w3 : (q == 1 ? a.off_b2 : a.off_b1)) + h, s[i], nullptr);
+            }
         return;
     }
     const bool second = b < n2;
@@ -1589,7 +1595,7 @@ bool sur_whole(const SurDev &s)
 }
 
 // bytes of one batch tile's X, A1, dZ2 and dZ1 and its partial sums
-size_t sur_tile_bytes(int K, int H) { return (size_t)BT * (up16(K) + 3 * H) * 2 + 12 * (size_t)H + 16; }
+size_t sur_tile_bytes(int K, int H) { return (size_t)BT * (up16(K) + 3 * H) * 2 + 12 * (size_t)H * BT + 4 * BT + 8; }
 
 namespace {
 
@@ -1647,8 +1653,8 @@ cudaError_t whole_step(const SurDev &s, NetArgs a, const AdamStep *step, float *
     a.dZ2t = take((size_t)BT * s.H * 2);
     a.dZ1t = take((size_t)BT * s.H * 2);
     a.part_loss = reinterpret_cast<double *>(take(8));
-    a.part = reinterpret_cast<float *>(take(12 * (size_t)s.H));
-    a.part_dy = reinterpret_cast<float *>(take(4));
+    a.cols = reinterpret_cast<float *>(take(12 * (size_t)s.H * BT));
+    a.dy = reinterpret_cast<float *>(take(4 * BT));
     rows_kernel<true><<<T, ROWS_THREADS, rows_plan(s.K, s.H).bytes, st>>>(a);
     GradArgs g{};
     g.n = a.n;
@@ -1661,8 +1667,8 @@ cudaError_t whole_step(const SurDev &s, NetArgs a, const AdamStep *step, float *
     g.A1t = a.A1t;
     g.dZ2t = a.dZ2t;
     g.dZ1t = a.dZ1t;
-    g.part = a.part;
-    g.part_dy = a.part_dy;
+    g.cols = a.cols;
+    g.dy = a.dy;
     g.part_loss = a.part_loss;
     g.p = s.p;
     g.g = s.g;
@@ -1677,7 +1683,7 @@ cudaError_t whole_step(const SurDev &s, NetArgs a, const AdamStep *step, float *
     g.W1b = s.W1b;
     g.W2b = s.W2b;
     g.err = s.err;
-    grads_kernel<<<grad_tiles(s.H, s.H) + grad_tiles(s.H, Kp) + 1, GRADS_THREADS, GRADS_SMEM, st>>>(g);
+    grads_kernel<<<grad_tiles(s.H, s.H) + grad_tiles(s.H, Kp) + vector_ctas(s.H), GRADS_THREADS, GRADS_SMEM, st>>>(g);
     return cudaGetLastError();
 }
 
