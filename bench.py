@@ -1104,7 +1104,7 @@ def _gradient_result(S, reps):
     achieved = ADJ_BYTES_PER_UPDATE * upd / (t / 1e3) / 1e9
     return {"workload": f"gradient-{gs.nx}x{gs.nz}-S{S}", "shots": S, "nt": nt, "ms": t,
             "point_steps": upd,
-            "roofline": {"kernel": "adjoint path (on-chip forward with history, adj_step2_kernel)",
+            "roofline": {"kernel": "adjoint path (on-chip forward with history, adj_group_kernel)",
                          "bound": "hbm", "achieved": achieved, "peak": peak, "peak_kind": peak_kind,
                          "unit": "GB/s", "frac": achieved / peak, "bytes_per_point_step": ADJ_BYTES_PER_UPDATE}}
 
