@@ -8,6 +8,8 @@
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
+#include <utility>
+
 #include "internal.cuh"
 
 namespace empso {
@@ -743,13 +745,17 @@ rank_corr_kernel(const double *__restrict__ fk, const int *__restrict__ rows,
 
 // mean and standard deviation of the filled replay targets, on one cluster of
 // STATS_C CTAs (FP64 sums run at 1/64 of the FP32 rate: one CTA took 14 us for
-// 6144 targets), summed in a fixed order
+// 6144 targets), summed in a fixed order.  Distributed shared memory may be
+// written only once its CTA has started: every CTA arrives at the cluster's
+// barrier on entry and waits there before it stores to CTA 0 (the wait falls
+// under the sums; with few targets the other CTAs reach their stores at once).
 constexpr int STATS_C = 8;
 __global__ void __cluster_dims__(STATS_C, 1, 1) __launch_bounds__(512)
 stats_kernel(const float *__restrict__ ybuf, const int *count, int have_host, int cap, float *stats)
 {
     __shared__ double s1[16], s2[16], c1[STATS_C], c2[STATS_C];
     cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    auto started = cluster.barrier_arrive();
     const int n = min(have_host >= 0 ? have_host : *count, cap);
     double a = 0.0, b = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += STATS_C * blockDim.x) {
@@ -767,6 +773,7 @@ stats_kernel(const float *__restrict__ ybuf, const int *count, int have_host, in
         s2[threadIdx.x >> 5] = b;
     }
     __syncthreads();
+    cluster.barrier_wait(std::move(started));
     if (threadIdx.x == 0) {
         a = b = 0.0;
         for (int w = 0; w < (int)blockDim.x / 32; ++w) {
