@@ -332,13 +332,16 @@ __device__ bool run_instance(const GridDev &g, const Inst &in, float *bufA, floa
     const bool has_rec = r0 < rec_e;
     Corners rc{};
     if (has_rec) rc = bilinear(in.rec[r0].x, in.rec[r0].y, g);
-    float accf = 0.f;                        // kept short in FP32, carried in FP64 every 32 steps
+    // The residual energy.  GF false: each square is formed and added in FP64.  GF
+    // true: in FP32 over 32 steps, as the on-chip kernel does, then carried in FP64.
+    float accf = 0.f;
     double acc = 0.0;
     auto record = [&](int r, int step, float d, float obs) {
         if (in.traces) in.traces[(size_t)(step - 1) * in.nrec + r] = d;
         if (in.dobs) {
             const float e = d - obs;
-            accf = fmaf(e, e, accf);
+            if (GF) accf = fmaf(e, e, accf);
+            else acc += (double)e * (double)e;
         }
     };
     if (!group_barrier(count, target, n, s_fail)) return false;
