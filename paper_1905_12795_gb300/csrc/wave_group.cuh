@@ -333,14 +333,16 @@ __device__ bool run_instance(const GridDev &g, const Inst &in, float *bufA, floa
     Corners rc{};
     if (has_rec) rc = bilinear(in.rec[r0].x, in.rec[r0].y, g);
     // The residual energy.  GF false: each square is formed and added in FP64.  GF
-    // true: in FP32 over 32 steps, as the on-chip kernel does, then carried in FP64.
+    // true: a thread's first receiver in FP32 over 32 steps, as the on-chip kernel
+    // does, then carried in FP64; its further receivers (groups of few CTAs) in FP64
+    // at once, so that an FP32 sum has 32 terms on every split.
     float accf = 0.f;
     double acc = 0.0;
     auto record = [&](int r, int step, float d, float obs) {
         if (in.traces) in.traces[(size_t)(step - 1) * in.nrec + r] = d;
         if (in.dobs) {
             const float e = d - obs;
-            if (GF) accf = fmaf(e, e, accf);
+            if (GF && r == r0) accf = fmaf(e, e, accf);
             else acc += (double)e * (double)e;
         }
     };

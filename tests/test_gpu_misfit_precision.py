@@ -1,6 +1,6 @@
 """Misfits of the plain streaming kernel (order 16, mixed orders, the
 allocation-free entry point): squares of the FP32 residuals and their sums are
-held in FP64, so residuals whose squares leave FP32's range keep a finite
+held in FP64 (the L2 kernel's in FP32 over 32 steps of one receiver), so residuals whose squares leave FP32's range keep a finite
 misfit, and no split of the GPU changes it by more than FP64 rounding."""
 import numpy as np
 import pytest
@@ -80,3 +80,22 @@ def test_allocation_free_misfit_keeps_large_residuals(B, order):
                           torch.full((n,), BIG, device="cuda"), mis)
     want = 0.5 * n * BIG * BIG
     assert abs(mis.item() - want) <= TOL * want
+
+
+def test_l2_misfit_sums_32_steps_of_one_receiver_in_fp32(B):
+    """The L2 kernel's FP32 sums: 32 squares of 6e36 fit FP32, 64 do not, so no
+    thread may add two receivers into one (64 shots of 1500 receivers give a
+    thread two)."""
+    nrec, S, c2 = 1500, 64, 6e36
+    grids, rec, xz = _setup(B, [8], nrec, S)
+    ctx = B.Context(grids, rec)
+    nt = ctx.grid_info(0)[1]
+    ctx.set_kernel(3)
+    big = float(np.float32(np.sqrt(c2)))
+    mis = torch.zeros(1, dtype=torch.float64, device="cuda")
+    ctx.eval_models(torch.full((1, 41, 61), 2000.0, device="cuda"), B.make_shots(xz, [0] * S, [nrec] * S),
+                    torch.full((S, nt, nrec), big, device="cuda"), mis)
+    assert ctx.last_launch()[0] == 3 and nt > 64
+    want = 0.5 * S * nt * nrec * big * big
+    assert abs(mis.item() - want) <= 32 * 2.0 ** -24 * want       # 32 FP32 additions
+    ctx.close()
