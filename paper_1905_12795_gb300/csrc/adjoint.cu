@@ -546,6 +546,8 @@ __device__ __forceinline__ void sweep_adjoint(const GridDev &g, const AdjInst &i
 {
     constexpr int N = Window<R>::N, XG = XRow<R>::XG, ZERO = XRow<R>::ZERO, LEN = XRow<R>::LEN, O = 4 * XG;
     const int lane = threadIdx.x & 31, NQ = g.NQ;
+    // (32-bit byte offsets: a grid of 4 GB and more does not fit the shared memory of
+    // adj_group_split, whose threads hold their whole run there)
     const unsigned pb = (unsigned)p4 * 16u;
     unsigned o_st = ((unsigned)(j0 + HALO) * (unsigned)p4 + HALO4 + q) * 16u;
     unsigned o_pf = o_st + PF * pb, o_w = o_st + (R + PF) * pb, o_ez = (unsigned)(j0 + HALO + PF) * 4u;

@@ -168,6 +168,7 @@ cudaError_t launch_vel_to_field(const GridDev &g, const float *vel, int M, float
 constexpr int WAVE_MAX_CTAS = 4096;      // co-resident CTAs of any device
 struct WaveSplit {
     int flight, group;
+    bool wide;                           // buffers of 4 GB or more: 64-bit byte offsets
 };
 WaveSplit wave_split(const GridDev *const *grids, int n_grids, int R, long long n_inst, long long by_l2,
                      bool hist = false);

@@ -22,18 +22,19 @@ namespace empso {
 
 namespace {
 
-template <int RF, bool HIST>
+template <int RF, bool HIST, bool WIDE = false>
 __global__ void __launch_bounds__(WAVE_THREADS, GroupCtas<RF>::v)
 wave_kernel(const GridDev *__restrict__ grids, const Inst *__restrict__ insts, int n_inst, int group, int *ws,
             float *slots, long long slot_floats, int *err, double *partial)
 {
-    group_cta<RF, false, HIST>(grids, insts, n_inst, group, ws, slots, slot_floats, err, partial);
+    group_cta<RF, false, HIST, WIDE>(grids, insts, n_inst, group, ws, slots, slot_floats, err, partial);
 }
 
 // (the history only at radius 8: the gradients of the other orders run their
 // forward pass on the cluster kernels or per step)
-WaveFn wave_fn(int R, bool hist = false)
+WaveFn wave_fn(int R, bool hist, bool wide)
 {
+    if (wide) return hist ? (R == 8 ? wave_kernel<8, true, true> : nullptr) : wave_kernel<0, false, true>;
     if (hist) return R == 8 ? wave_kernel<8, true> : nullptr;
     if (R == 8) return wave_kernel<8, false>;
     if (R == 4) return wave_kernel<4, false>;
@@ -45,14 +46,14 @@ WaveFn wave_fn(int R, bool hist = false)
 
 WaveSplit wave_split(const GridDev *const *grids, int n_grids, int R, long long n_inst, long long by_l2, bool hist)
 {
-    return group_split(grids, n_grids, group_max_ctas(wave_fn(R, hist)), n_inst, by_l2);
+    return group_split(grids, n_grids, group_max_ctas(wave_fn(R, hist, group_wide(grids, n_grids))), n_inst, by_l2);
 }
 
 cudaError_t launch_wave(int R, const GridDev *grids_dev, const Inst *insts, int n_inst, const WaveSplit &s,
                         void *ws, float *slots, long long slot_floats, int *err, double *partial, cudaStream_t st,
                         bool hist)
 {
-    return launch_groups(wave_fn(R, hist), grids_dev, insts, n_inst, s, ws, slots, slot_floats, err, partial, st);
+    return launch_groups(wave_fn(R, hist, s.wide), grids_dev, insts, n_inst, s, ws, slots, slot_floats, err, partial, st);
 }
 
 // misfit[p] = sum_s weight_s partial[p][s] in fixed shot order; non-finite

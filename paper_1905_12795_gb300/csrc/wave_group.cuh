@@ -121,6 +121,14 @@ __device__ __forceinline__ void cp_async16(void *sdst, const void *gsrc)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gsrc) : "memory");
 }
 
+// a byte offset into a buffer
+template <bool WIDE> struct ByteOffset {
+    using type = unsigned;
+};
+template <> struct ByteOffset<true> {
+    using type = unsigned long long;
+};
+
 // num / d for d >= 1: a reciprocal after one Newton step on the hardware's
 // approximation, and the quotient corrected by its exact remainder (Markstein's
 // method, which gives the correctly rounded quotient); d = 1 returns num.
@@ -153,27 +161,32 @@ __device__ __forceinline__ float2 quot2(float2 num, float2 d)
 // GF false: u^{n+1} = [a lap + (2 u^n - (1 - t) u^{n-1})] / (1 + t), the scheme
 // as written.  GF true: u^{n+1} = g (u^n - u^{n-1}) + u^{n-1} + (a g / 2) lap
 // with g = 2 / (1 + t), fewer operations and a tenth of the rounding error.
-template <int R, bool GF, bool HIST>
+//
+// Byte offsets into a buffer are 32 bits wide (64-bit ones cost an addition per
+// access: 33 against 31 us a step, order 16, 16 instances on the 1041 x 421 grid).
+// WIDE, for buffers of 4 GB and more: 64 bits.
+template <int R, bool GF, bool HIST, bool WIDE>
 __device__ __forceinline__ void sweep_run(const GridDev &g, const float4 *cur, float4 *prev, float4 *hist,
                                           const float4 *__restrict__ a4, int p4, int q, int j0, int len, bool act,
                                           int lmax, float4 *xb, const float *cx, const float *cz, float cres,
                                           int s_i0, int s_j0, const float *sw, float rn)
 {
     constexpr int N = Window<R>::N, XG = XRow<R>::XG, ZERO = XRow<R>::ZERO, LEN = XRow<R>::LEN;
+    using Ofs = typename ByteOffset<WIDE>::type;
     const int lane = threadIdx.x & 31, NQ = g.NQ;
-    // byte offsets into the buffers (a buffer holds less than 4 GB): row k's own
-    // group, the ones requested in row k, and the edge group
-    const unsigned pb = (unsigned)p4 * 16u;
-    unsigned o_st = ((unsigned)(j0 + HALO) * (unsigned)p4 + HALO4 + q) * 16u;
-    unsigned o_um = o_st + PF * pb, o_w = o_st + (R + PF) * pb, o_ez = (unsigned)(j0 + HALO + PF) * 4u;
-    auto ld = [](const char *p, unsigned o) { return *reinterpret_cast<const float4 *>(p + o); };
-    auto ldg = [](const char *p, unsigned o) { return __ldg(reinterpret_cast<const float4 *>(p + o)); };
+    // byte offsets into the buffers: row k's own group, the ones requested in row k,
+    // and the edge group
+    const Ofs pb = (Ofs)p4 * 16u;
+    Ofs o_st = ((Ofs)(j0 + HALO) * (Ofs)p4 + HALO4 + q) * 16u;
+    Ofs o_um = o_st + PF * pb, o_w = o_st + (R + PF) * pb;
+    unsigned o_ez = (unsigned)(j0 + HALO + PF) * 4u;
+    auto ld = [](const char *p, Ofs o) { return *reinterpret_cast<const float4 *>(p + o); };
+    auto ldg = [](const char *p, Ofs o) { return __ldg(reinterpret_cast<const float4 *>(p + o)); };
     // the edge group this lane fetches for the warp: the run of lane 0 or 31
     const bool left = lane < XG, edge = left || lane >= 32 - XG;
     const int src = left ? 0 : 31;
     const int qe = __shfl_sync(0xffffffffu, q, src), je = __shfl_sync(0xffffffffu, j0, src);
-    unsigned o_e =
-        ((unsigned)(je + HALO) * (unsigned)p4 + HALO4 + qe + (left ? lane - XG : lane - (32 - XG) + 1)) * 16u;
+    Ofs o_e = ((Ofs)(je + HALO) * (Ofs)p4 + HALO4 + qe + (left ? lane - XG : lane - (32 - XG) + 1)) * 16u;
     float4 *eslot = xb + (left ? lane : lane + 2 * XG), *own = xb + XG + lane;
     // where the x-neighbours are
     const float4 *x_l = xb + (q >= 1 ? XG + lane - 1 : ZERO), *x_r = xb + (q + 1 < NQ ? XG + lane + 1 : ZERO);
@@ -293,7 +306,7 @@ __device__ __forceinline__ void sweep_run(const GridDev &g, const float4 *cur, f
 
 // CTA `rank` of a group of n runs its part of instance `in`; bufA / bufB are
 // the group's slot.  False when a barrier gave up.
-template <int R, bool GF, bool HIST>
+template <int R, bool GF, bool HIST, bool WIDE>
 __device__ bool run_instance(const GridDev &g, const Inst &in, float *bufA, float *bufB, float4 *xrows,
                              float (*samples)[WAVE_THREADS], int rank, int n, unsigned *count, unsigned &target,
                              int *s_fail, double *red, double *gpart, double *partial)
@@ -371,7 +384,7 @@ __device__ bool run_instance(const GridDev &g, const Inst &in, float *bufA, floa
             const int q = min(item, items - 1) % NQ, seg = min(item, items - 1) / NQ;
             const int j0 = (int)((long long)seg * g.NZ / nseg), j1 = (int)((long long)(seg + 1) * g.NZ / nseg);
             const int len = j1 - j0;
-            sweep_run<R, GF, HIST>(g, reinterpret_cast<const float4 *>(cur), reinterpret_cast<float4 *>(prev),
+            sweep_run<R, GF, HIST, WIDE>(g, reinterpret_cast<const float4 *>(cur), reinterpret_cast<float4 *>(prev),
                          HIST ? reinterpret_cast<float4 *>(in.hist + (size_t)(step + 1) * g.field) : nullptr, a4, p4,
                          q, j0, len, act, __reduce_max_sync(0xffffffffu, len), xb, cx,
                          cz, cres, s_i0, s_j0, sw, rn);
@@ -427,8 +440,9 @@ template <int RF> struct GroupCtas {
     static constexpr int v = RF == 0 || RF == 8 ? 2 : 3;
 };
 
-// a CTA's whole work; RF: the radius of every grid of the launch (0: per instance)
-template <int RF, bool GF, bool HIST>
+// a CTA's whole work; RF: the radius of every grid of the launch (0: per instance);
+// WIDE: some grid's buffer holds 4 GB or more
+template <int RF, bool GF, bool HIST, bool WIDE>
 __device__ __forceinline__ void group_cta(const GridDev *__restrict__ grids, const Inst *__restrict__ insts, int n_inst,
                                           int group, int *ws, float *slots, long long slot_floats, int *err,
                                           double *partial)
@@ -463,12 +477,12 @@ __device__ __forceinline__ void group_cta(const GridDev *__restrict__ grids, con
         const GridDev &g = sg;
         float *bufB = bufA + g.field;
         auto run = [&](auto r) {
-            return run_instance<decltype(r)::value, GF, HIST>(g, in, bufA, bufB, xrows, samples, rank, group, count,
+            return run_instance<decltype(r)::value, GF, HIST, WIDE>(g, in, bufA, bufB, xrows, samples, rank, group, count,
                                                              target, &s_fail, red, gpart, partial);
         };
         bool ok;
         if constexpr (RF != 0) ok = run(Radius<RF>{});
-        else if (g.R == 8) ok = run(Radius<8>{});
+        else if (!GF && g.R == 8) ok = run(Radius<GF ? 4 : 8>{});     // (GF: the L2 kernel, radius up to 4)
         else if (g.R == 4) ok = run(Radius<4>{});
         else if (g.R == 2) ok = run(Radius<2>{});
         else ok = run(Radius<1>{});
@@ -497,6 +511,14 @@ inline int group_max_ctas(WaveFn fn)
     return memo[{dev, fn}] = std::min(sms * n, WAVE_MAX_CTAS);
 }
 
+// does some grid's buffer need 64-bit byte offsets?
+inline bool group_wide(const GridDev *const *grids, int n_grids)
+{
+    bool wide = false;
+    for (int i = 0; i < n_grids; ++i) wide = wide || 4 * grids[i]->field > 1LL << 32;
+    return wide;
+}
+
 // Instances in flight and CTAs per instance: the split of the co-resident CTAs
 // with the least estimated time, rounds of instances x rows a thread sweeps
 // (plus RUN_EXTRA rows' worth for the window it loads first and the step
@@ -507,6 +529,7 @@ inline WaveSplit group_split(const GridDev *const *grids, int n_grids, int ctas,
 {
     constexpr int RUN_EXTRA = 10;
     WaveSplit best{};
+    best.wide = group_wide(grids, n_grids);
     const long long most = std::max<long long>(1, std::min<long long>({n_inst, by_l2, (long long)ctas}));
     double cost = 0.0;
     if (ctas > 0 && fixed > 0) {

@@ -16,16 +16,17 @@ namespace empso {
 
 namespace {
 
-template <int RF, bool HIST>
+template <int RF, bool HIST, bool WIDE = false>
 __global__ void __launch_bounds__(WAVE_THREADS, GroupCtas<RF>::v)
 wave_l2_kernel(const GridDev *__restrict__ grids, const Inst *__restrict__ insts, int n_inst, int group, int *ws,
                float *slots, long long slot_floats, int *err, double *partial)
 {
-    group_cta<RF, true, HIST>(grids, insts, n_inst, group, ws, slots, slot_floats, err, partial);
+    group_cta<RF, true, HIST, WIDE>(grids, insts, n_inst, group, ws, slots, slot_floats, err, partial);
 }
 
-WaveFn l2_fn(int R, bool hist)
+WaveFn l2_fn(int R, bool hist, bool wide)
 {
+    if (wide) return hist ? wave_l2_kernel<0, true, true> : wave_l2_kernel<0, false, true>;
     if (hist) {
         if (R == 4) return wave_l2_kernel<4, true>;
         if (R == 2) return wave_l2_kernel<2, true>;
@@ -52,7 +53,7 @@ bool l2_fits(const GridDev &g, int C, int nrec, size_t limit)
 WaveSplit l2_split(const GridDev *const *grids, int n_grids, int R, long long n_inst, long long by_l2, int C, int sms,
                    bool hist)
 {
-    const int ctas = group_max_ctas(l2_fn(R, hist));
+    const int ctas = group_max_ctas(l2_fn(R, hist, group_wide(grids, n_grids)));
     return group_split(grids, n_grids, ctas, n_inst, by_l2, C > 0 ? C * std::max(1, ctas / sms) : 0);
 }
 
@@ -60,7 +61,7 @@ cudaError_t launch_wave_l2(int R, const GridDev *grids_dev, const Inst *insts, i
                            void *ws, float *slots, long long slot_floats, int *err, double *partial, cudaStream_t st,
                            bool hist)
 {
-    return launch_groups(l2_fn(R, hist), grids_dev, insts, n_inst, s, ws, slots, slot_floats, err, partial, st);
+    return launch_groups(l2_fn(R, hist, s.wide), grids_dev, insts, n_inst, s, ws, slots, slot_floats, err, partial, st);
 }
 
 }  // namespace empso
