@@ -346,16 +346,19 @@ __device__ bool run_instance(const GridDev &g, const Inst &in, float *bufA, floa
     Corners rc{};
     if (has_rec) rc = bilinear(in.rec[r0].x, in.rec[r0].y, g);
     // The residual energy.  GF false: each square is formed and added in FP64.  GF
-    // true: a thread's first receiver in FP32 over 32 steps, as the on-chip kernel
-    // does, then carried in FP64; its further receivers (groups of few CTAs) in FP64
-    // at once, so that an FP32 sum has 32 terms on every split.
+    // true: 32 squares are added in FP32, as the on-chip kernel does, then carried in
+    // FP64: 32 steps of a thread with one receiver, fewer where a thread has more
+    // (groups of few CTAs).  (FP64 sums for a thread's further receivers, in this loop:
+    // 0.5 to 3 % on the 921 x 301 grid, whose threads have none.)
+    const int per = (rec_e - rec_b + WAVE_THREADS - 1) / WAVE_THREADS;    // receivers of a thread
+    const int flush = per <= 1 ? 31 : (per <= 2 ? 15 : (per <= 4 ? 7 : (per <= 8 ? 3 : (per <= 16 ? 1 : 0))));
     float accf = 0.f;
     double acc = 0.0;
     auto record = [&](int r, int step, float d, float obs) {
         if (in.traces) in.traces[(size_t)(step - 1) * in.nrec + r] = d;
         if (in.dobs) {
             const float e = d - obs;
-            if (GF && r == r0) accf = fmaf(e, e, accf);
+            if (GF) accf = fmaf(e, e, accf);
             else acc += (double)e * (double)e;
         }
     };
@@ -397,7 +400,7 @@ __device__ bool run_instance(const GridDev &g, const Inst &in, float *bufA, floa
                        rc.w[3] * samples[3][tid],
                    in.dobs ? samples[4][tid] : 0.f);
         }
-        if ((step & 31) == 0) {
+        if (GF && (step & flush) == 0) {
             acc += (double)accf;
             accf = 0.f;
         }
