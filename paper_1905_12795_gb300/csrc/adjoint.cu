@@ -641,7 +641,7 @@ __device__ __forceinline__ void sweep_adjoint(const GridDev &g, const AdjInst &i
             const float2 z = splat2(ez[kk]);
             const float2 t01 = __fadd2_rn(lo2(ex), z), t23 = __fadd2_rn(hi2(ex), z);
             const float2 d01 = __fadd2_rn(one, t01), d23 = __fadd2_rn(one, t23);
-            const float2 f01 = quot2(one, d01), f23 = quot2(one, d23);
+            const float2 f01 = quot2<true>(one, d01), f23 = quot2<true>(one, d23);
             const float2 h01 = __fmul2_rn(__fadd2_rn(t01, mone), f01), h23 = __fmul2_rn(__fadd2_rn(t23, mone), f23);
             m01 = __fadd2_rn(__ffma2_rn(h01, lo2(a2), __ffma2_rn(__fmul2_rn(two, f01), lo2(a1), o01)), j01);
             m23 = __fadd2_rn(__ffma2_rn(h23, hi2(a2), __ffma2_rn(__fmul2_rn(two, f23), hi2(a1), o23)), j23);

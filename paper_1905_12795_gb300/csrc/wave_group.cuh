@@ -129,11 +129,19 @@ template <> struct ByteOffset<true> {
     using type = unsigned long long;
 };
 
-// num / d for d >= 1: a reciprocal after one Newton step on the hardware's
-// approximation, and the quotient corrected by its exact remainder (Markstein's
-// method, which gives the correctly rounded quotient); d = 1 returns num.
-// With the library's division and reciprocal in their place the damping layer's
-// rows took twice the time of the others (60 cells: 33.6 us a step against 21.6)
+// num / d for 1 <= d < 4096: a reciprocal after one Newton step on the hardware's
+// approximation, and the quotient corrected by its remainder (Markstein's method:
+// correctly rounded where the remainder is exact, for |num| from 2^-90 up; below, the
+// remainder may be subnormal, and the error within half a last place and 2^-150);
+// d = 1 returns num, and infinities and not-a-numbers stay what they are (the
+// remainder of an infinity is not a number: the larger of it and -MOST is -MOST, and
+// its product added to the infinity leaves that).  With the compiler's division in its
+// place the damping layer's rows took twice the time of the others (60 cells, order 16,
+// 16 instances on the 1041 x 421 grid: 33.6 us a step against 21.6); correctly
+// rounded below 2^-90 too, by scaling, those rows cost a fifth more, and the waves'
+// first traces, where such numbers are, run ahead of them through the whole grid.
+// FINITE: num is known to be.
+template <bool FINITE = false>
 __device__ __forceinline__ float2 quot2(float2 num, float2 d)
 {
     float2 y;
@@ -142,7 +150,10 @@ __device__ __forceinline__ float2 quot2(float2 num, float2 d)
     const float2 nd = __fmul2_rn(splat2(-1.f), d);
     y = __ffma2_rn(y, __ffma2_rn(nd, y, splat2(1.f)), y);
     const float2 q = __fmul2_rn(num, y);
-    return __ffma2_rn(__ffma2_rn(nd, q, num), y, q);
+    float2 r = __ffma2_rn(nd, q, num);
+    constexpr float MOST = 0x1.fffffep127f;
+    if (!FINITE) r = f2(fmaxf(r.x, -MOST), fmaxf(r.y, -MOST));
+    return __ffma2_rn(r, y, q);
 }
 
 // One step of one run: rows j0 .. j0 + len - 1 of column group q, the whole
