@@ -413,8 +413,10 @@ empso_status empso_read_timing(empso_ctx *ctx, double *ms3);
  * All calls share the array and it keeps the last call's contents (the call
  * clears what must start at zero itself); calls that overlap on the GPU -
  * different streams, or different host threads, on one device - race on it
- * and must be serialised by the caller.  Errors: INVALID_ARG, UNSUPPORTED,
- * CUDA_ERROR; message in empso_last_error(NULL). */
+ * and must be serialised by the caller.  There is no status word as a context
+ * has one: when a bounded wait inside the modelling kernel gives up, the misfits
+ * of the models it leaves unfinished are +inf.  Errors: INVALID_ARG,
+ * UNSUPPORTED, CUDA_ERROR; message in empso_last_error(NULL). */
 empso_status eval_models_noalloc(const empso_grid *grid, const float *rec_xz,
                                  int32_t nrec_total, const float *vel, int32_t M,
                                  const empso_shot *shots, int32_t S,

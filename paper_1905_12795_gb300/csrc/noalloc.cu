@@ -52,7 +52,6 @@ struct Layout {
     float *weights;
     Inst *insts;
     double *partial;
-    int *err;                  // status word of the launch's bounded waits
     float *fields;
     float *slots;
     size_t used;
@@ -80,7 +79,6 @@ Layout carve(unsigned char *base, const GridDev &g, int S, int nrec_total, int M
     L.weights = reinterpret_cast<float *>(take(sizeof(float) * S));
     L.insts = reinterpret_cast<Inst *>(take(sizeof(Inst) * (size_t)M * S));
     L.partial = reinterpret_cast<double *>(take(sizeof(double) * (size_t)M * S));
-    L.err = reinterpret_cast<int *>(take(sizeof(int)));
     L.fields = reinterpret_cast<float *>(take(sizeof(float) * (size_t)M * g.field));
     L.slots = reinterpret_cast<float *>(take(sizeof(float) * 2 * (size_t)g.field * n_slots));
     L.used = o;
@@ -219,7 +217,9 @@ extern "C" empso_status eval_models_noalloc(const empso_grid *grid, const float 
         (e = launch_grid_tables(p.g, L.ex, L.ez, L.wavelet, L.Wx, L.Wz, grid->vmax, grid->f0, st)) !=
             cudaSuccess ||
         (e = launch_vel_to_field(p.g, vel, M, L.fields, p.g.field, st)) != cudaSuccess ||
-        (e = launch_wave(g.R, L.grid, L.insts, (int)n_inst, split, ws, L.slots, 2 * p.g.field, L.err, L.partial,
+        // (no status word: a wait that gives up leaves its instances' misfits not a number,
+        // which the sums below turn into +inf)
+        (e = launch_wave(g.R, L.grid, L.insts, (int)n_inst, split, ws, L.slots, 2 * p.g.field, nullptr, L.partial,
                          st)) != cudaSuccess ||
         (e = launch_finalize(L.partial, L.weights, M, S, misfit, nullptr, st)) != cudaSuccess)
         return nfail(EMPSO_CUDA_ERROR, cudaGetErrorString(e));

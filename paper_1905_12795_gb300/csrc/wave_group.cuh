@@ -502,7 +502,14 @@ __device__ __forceinline__ void group_cta(const GridDev *__restrict__ grids, con
         else ok = run(Radius<1>{});
         if (!ok) break;
     }
-    if (threadIdx.x == 0 && s_fail) atomicExch(err, EMPSO_TIMEOUT);
+    if (threadIdx.x == 0 && s_fail) {
+        // a group that gave up also takes what is left of the queue: no instance keeps
+        // what an earlier launch left as its misfit
+        if (rank == 0)
+            for (int q = atomicAdd(ws, 1); q < n_inst; q = atomicAdd(ws, 1))
+                partial[insts[q].out] = __longlong_as_double(0x7ff8000000000000LL);
+        if (err) atomicExch(err, EMPSO_TIMEOUT);
+    }
 }
 
 using WaveFn = void (*)(const GridDev *, const Inst *, int, int, int *, float *, long long, int *, double *);
