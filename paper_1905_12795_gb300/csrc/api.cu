@@ -1897,15 +1897,16 @@ empso_status empso_autotune(empso_ctx *ctx, const float *particles, int32_t P,
     cudaEvent_t e0, e1;
     CK(ctx, cudaEventCreate(&e0));
     CK(ctx, cudaEventCreate(&e1));
-    // candidates: the streaming kernel, every cluster size and rows-per-thread
-    // shape of the on-chip one, and the usual cluster sizes of the L2 one
-    // (only those of the selected kind when a kind is selected)
+    // candidates: the streaming kernel, every cluster size and run length that the
+    // planner chooses among for the on-chip one (its own shape is one of them), and the
+    // usual SMs per instance of the L2 one (only those of the selected kind when a kind
+    // is selected)
     const int only = ctx->kernel_kind;
     std::vector<empso_ctx::Tuned> cand;
     if (only == EMPSO_KERNEL_AUTO || only == EMPSO_KERNEL_STREAMING) cand.push_back({EMPSO_KERNEL_STREAMING, 0, 0});
     if (only == EMPSO_KERNEL_AUTO || only == EMPSO_KERNEL_RESIDENT)
         for (int C = 1; C <= 16; ++C)
-            for (const int rows : RESIDENT_RUNS) cand.push_back({EMPSO_KERNEL_RESIDENT, C, rows});
+            for (const int rows : RESIDENT_RUNS_EST) cand.push_back({EMPSO_KERNEL_RESIDENT, C, rows});
     if (only == EMPSO_KERNEL_AUTO || only == EMPSO_KERNEL_CLUSTER_L2)
         for (int C : {0, 4, 8, 10, 12, 16}) cand.push_back({EMPSO_KERNEL_CLUSTER_L2, C, 0});   // 0: the planner's split
     float best = 1e30f;
