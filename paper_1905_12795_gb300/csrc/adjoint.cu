@@ -842,6 +842,8 @@ AdjGroupFn adj_group_fn(int R)
     return R == 2 ? adj_group_kernel<2> : adj_group_kernel<1>;
 }
 size_t adj_group_smem(int rows) { return sizeof(float4) * 3 * (size_t)rows * WAVE_THREADS; }
+// a CTA's share of an SM's shared memory, less its static part and the system's 1 KB
+size_t adj_group_room(size_t smem_optin) { return smem_optin / ADJ_CTAS - (12u << 10); }
 
 // residual e_n = R u^{n+1} - d_obs,n (one block per instance), u^{n+1} in the
 // rotating slots of the per-step forward pass
@@ -1027,6 +1029,15 @@ cudaError_t launch_adj_residual(const GridDev &g, const AdjInst *insts, int n_in
     return cudaGetLastError();
 }
 
+// Opts the persistent backward pass of radius R into the most shared memory any
+// split takes, on the current device: once per context, as the limit is the
+// kernel's and another thread's gradient may be between its split and its launch.
+cudaError_t adj_group_configure(int R, size_t smem_optin)
+{
+    return cudaFuncSetAttribute(adj_group_fn(R), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)adj_group_room(smem_optin));
+}
+
 // Instances in flight and sweeping CTAs each (one more scatters) of the
 // persistent backward pass: the least estimated time among the splits whose
 // threads' rows fit shared memory; group 0 when none does, or when up to radius
@@ -1043,8 +1054,7 @@ AdjSplit adj_group_split(const GridDev &g, long long n_inst, size_t smem_optin)
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return best;
     const int per = ADJ_CTAS, ctas = std::min(sms * per, WAVE_MAX_CTAS);
-    // an SM's shared memory, less each CTA's static part and the system's 1 KB
-    const size_t room = smem_optin / per - (12u << 10);
+    const size_t room = adj_group_room(smem_optin);
     double cost = 0.0;
     for (long long f = 1; f <= std::min<long long>(n_inst, ctas / 2); ++f) {
         const int n = (int)(ctas / f) - 1, nseg = std::min(g.NZ, n * WAVE_THREADS / g.NQ);
@@ -1062,9 +1072,7 @@ AdjSplit adj_group_split(const GridDev &g, long long n_inst, size_t smem_optin)
     // (the CTAs of a group wait for one another: all must be resident)
     int fit = 0;
     if (best.group &&
-        (cudaFuncSetAttribute(adj_group_fn(g.R), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)adj_group_smem(best.rows)) != cudaSuccess ||
-         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, adj_group_fn(g.R), WAVE_THREADS, adj_group_smem(best.rows)) !=
+        (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, adj_group_fn(g.R), WAVE_THREADS, adj_group_smem(best.rows)) !=
              cudaSuccess ||
          fit < per)) {
         cudaGetLastError();
@@ -1078,8 +1086,7 @@ cudaError_t launch_adj_group(const GridDev &g, const AdjInst *insts, int n_inst,
 {
     const AdjGroupFn fn = adj_group_fn(g.R);
     const size_t smem = adj_group_smem(s.rows);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) e = cudaMemsetAsync(ws, 0, sizeof(int) * WS_LINE * (1 + (size_t)s.flight), st);
+    const cudaError_t e = cudaMemsetAsync(ws, 0, sizeof(int) * WS_LINE * (1 + (size_t)s.flight), st);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];

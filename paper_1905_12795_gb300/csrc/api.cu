@@ -1036,6 +1036,8 @@ empso_status empso_create(const empso_grid *grids, int32_t ngrids, const float *
             if ((rc = ck(stream_configure(R, ctx->smem_optin), "streaming kernel attributes")))
                 return bail(rc);
         }
+        for (int R : {1, 2, 4, 8})
+            if ((rc = ck(adj_group_configure(R, ctx->smem_optin), "adjoint kernel attributes"))) return bail(rc);
         if ((rc = ck(cudaMalloc(&ctx->dev_err, sizeof(int)), "error word")) ||
             (rc = ck(cudaMemset(ctx->dev_err, 0, sizeof(int)), "error word")) ||
             (rc = ck(cudaMalloc(&ctx->nonfinite, 2 * sizeof(unsigned long long)), "counters")) ||

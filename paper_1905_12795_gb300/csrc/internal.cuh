@@ -132,6 +132,7 @@ cudaError_t launch_adj_backward(const GridDev &g, const AdjInst *insts, int n_in
 struct AdjSplit {
     int flight, group, rows;
 };
+cudaError_t adj_group_configure(int R, size_t smem_optin);
 AdjSplit adj_group_split(const GridDev &g, long long n_inst, size_t smem_optin);
 cudaError_t launch_adj_group(const GridDev &g, const AdjInst *insts, int n_inst, const AdjSplit &s, void *ws, int *err,
                              cudaStream_t st);
