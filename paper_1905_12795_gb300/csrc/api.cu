@@ -1343,8 +1343,9 @@ empso_status gradient_impl(empso_ctx *ctx, const float *vel, int M, const empso_
                     (ctx->kernel_kind == EMPSO_KERNEL_AUTO || ctx->kernel_kind == EMPSO_KERNEL_CLUSTER_L2);
     if (ctx->kernel_kind == EMPSO_KERNEL_CLUSTER_L2 && !l2)
         return fail(ctx, EMPSO_UNSUPPORTED, "gradient: the grid does not fit the L2 cluster kernel");
-    if (l2) split = l2_split(&gp, 1, g.R, I, by_l2, 0, ctx->sm_count, true);
-    if (g.R > MAX_R_FAST) split = wave_split(&gp, 1, g.R, I, by_l2, true);
+    // (the misfit alone runs the instantiation without the history: its own co-residency)
+    if (l2) split = l2_split(&gp, 1, g.R, I, by_l2, 0, ctx->sm_count, !forward_only);
+    if (g.R > MAX_R_FAST) split = wave_split(&gp, 1, g.R, I, by_l2, !forward_only);
     if ((l2 || g.R > MAX_R_FAST) && split.group < 1)
         return fail(ctx, EMPSO_CUDA_ERROR, "gradient: occupancy of the forward kernel");
     const AdjSplit back = adj_group_split(g, I, ctx->smem_optin);
