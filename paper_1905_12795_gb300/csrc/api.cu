@@ -86,7 +86,13 @@ struct empso_ctx {
     size_t stage_cap = 0;        // bytes
     cudaEvent_t stage_free = nullptr;
     int *counter = nullptr;
-    cudaMemPool_t pool = nullptr;         // stream-ordered workspace (low-pass taps)
+    // low-pass taps: a slab for the calls of one stream (the first that needs it),
+    // stream-ordered memory for larger tables and for other streams
+    std::mutex lp_mu;
+    float *lp_slab = nullptr;
+    bool lp_bound = false;
+    unsigned long long lp_stream = 0;     // the slab's stream (its id: a handle may be used again)
+    cudaMemPool_t pool = nullptr;
     unsigned char *wave_ws = nullptr;     // plain streaming kernel: queue, group barriers, partial sums
     size_t wave_ws_cap = 0;               // bytes
 
@@ -419,6 +425,10 @@ struct Models {
 // Instances of the L2-resident cluster kernel in flight are capped so that
 // their time levels and model fields fit this share of the 129 MB L2.
 constexpr long long L2_BUDGET_BYTES = 96LL << 20;
+
+// Low-pass workspace made with the context (16 shots of 461 receivers, 1414 outputs
+// with a 1 s window, take 6.5 MB of it).
+constexpr size_t LP_SLAB_BYTES = 8u << 20;
 
 struct Plan {
     int M = 0, S = 0;
@@ -904,6 +914,7 @@ void free_ctx(empso_ctx *c)
     cudaFree(c->stage_dev);
     cudaFree(c->counter);
     cudaFree(c->wave_ws);
+    cudaFree(c->lp_slab);
     if (c->pool) cudaMemPoolDestroy(c->pool);
     cudaFree(c->dev_err);
     cudaFree(c->nonfinite);
@@ -1100,7 +1111,8 @@ empso_status empso_create(const empso_grid *grids, int32_t ngrids, const float *
             (rc = ck(cudaMemset(ctx->pso_int, 0, sizeof(int) * (2 * p.P + 3)), "swarm ints")))
             return bail(rc);
     }
-    if ((rc = ck(cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking), "capture stream")) ||
+    if ((rc = ck(cudaMalloc(&ctx->lp_slab, LP_SLAB_BYTES), "low-pass workspace")) ||
+        (rc = ck(cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking), "capture stream")) ||
         (rc = ck(cudaEventCreateWithFlags(&ctx->chain_fork, cudaEventDisableTiming), "chain event")))
         return bail(rc);
     for (int i = 0; i < empso_ctx::MAX_CHAINS - 1; ++i)
@@ -1205,8 +1217,22 @@ empso_status empso_lowpass(empso_ctx *ctx, const float *in, int32_t S, int32_t n
     if (!lowpass_supported(dt_in, dt_out, half_width, ctx->smem_optin))
         return fail(ctx, EMPSO_UNSUPPORTED, "filter window too long for shared memory "
                                             "(half_width / dt_in too large)");
-    // the taps' workspace comes from the context's own pool in stream order, so
-    // that calls on several streams do not share it and a capture owns its own
+    cudaStream_t st = (cudaStream_t)stream;
+    const size_t need = lowpass_ws_floats(S, nrec, nt_out, dt_in, dt_out, half_width, ctx->sm_count);
+    unsigned long long id = 0;
+    CK(ctx, cudaStreamGetId(st, &id));
+    std::lock_guard<std::mutex> lock(ctx->lp_mu);
+    if (!ctx->lp_bound) {
+        ctx->lp_bound = true;
+        ctx->lp_stream = id;
+    }
+    if (id == ctx->lp_stream && sizeof(float) * need <= LP_SLAB_BYTES) {
+        CK(ctx, launch_lowpass(in, S, nt_in, nrec, dt_in, out, nt_out, dt_out, f_cut, half_width, ctx->lp_slab, need,
+                               ctx->sm_count, st));
+        return EMPSO_OK;
+    }
+    // from the context's own pool in stream order, so that calls on several streams
+    // do not share it and a capture owns its own
     if (!ctx->pool) {
         cudaMemPoolProps props = {};
         props.allocType = cudaMemAllocationTypePinned;
@@ -1216,8 +1242,6 @@ empso_status empso_lowpass(empso_ctx *ctx, const float *in, int32_t S, int32_t n
         uint64_t keep = 128ull << 20;       // bytes kept between calls
         CK(ctx, cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep));
     }
-    cudaStream_t st = (cudaStream_t)stream;
-    const size_t need = lowpass_ws_floats(S, nrec, nt_out, dt_in, dt_out, half_width, ctx->sm_count);
     float *ws = nullptr;
     const cudaError_t me = cudaMallocFromPoolAsync((void **)&ws, sizeof(float) * need, ctx->pool, st);
     if (me == cudaErrorMemoryAllocation) {
