@@ -477,7 +477,8 @@ empso_status empso_level_bounds(int32_t n_levels, const float *level_z,
  * band is about 3 / half_width Hz wide.  in and out must not overlap.
  * Workspace: 8 MB made with the context serve the first stream that filters;
  * larger tables of taps (up to 64 MB) and other streams take stream-ordered
- * memory of the context's.  Errors: INVALID_ARG, UNSUPPORTED (window of more
+ * memory of the context's.  A captured call's table stays with the graph, its
+ * clones and instantiations; the context outlives their launches.  Errors: INVALID_ARG, UNSUPPORTED (window of more
  * than the shared memory holds: half_width / dt_in too large), OOM. */
 empso_status empso_lowpass(empso_ctx *ctx, const float *in, int32_t S, int32_t nt_in,
                            int32_t nrec, double dt_in, float *out, int32_t nt_out,

@@ -8,6 +8,7 @@
 #include <fstream>
 #include <random>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <sstream>
@@ -65,6 +66,19 @@ struct GridHost {
     float4 *lw = nullptr;
 };
 
+// Device buffers that captured graphs hold: one stays with its graph, its clones
+// and instantiations until the last of them is destroyed, then another capture may
+// take it.  All are freed with the context.
+struct GraphBuffers {
+    std::mutex mu;
+    struct Buffer {
+        void *p;
+        size_t bytes;
+        bool taken;
+    };
+    std::vector<Buffer> all;
+};
+
 struct empso_ctx {
     int device = 0;
     int sm_count = 0;
@@ -93,6 +107,7 @@ struct empso_ctx {
     bool lp_bound = false;
     unsigned long long lp_stream = 0;     // the slab's stream (its id: a handle may be used again)
     cudaMemPool_t pool = nullptr;
+    std::shared_ptr<GraphBuffers> lp_graphs = std::make_shared<GraphBuffers>();   // captured calls' tables
     unsigned char *wave_ws = nullptr;     // plain streaming kernel: queue, group barriers, partial sums
     size_t wave_ws_cap = 0;               // bytes
 
@@ -915,6 +930,7 @@ void free_ctx(empso_ctx *c)
     cudaFree(c->counter);
     cudaFree(c->wave_ws);
     cudaFree(c->lp_slab);
+    for (auto &b : c->lp_graphs->all) cudaFree(b.p);
     if (c->pool) cudaMemPoolDestroy(c->pool);
     cudaFree(c->dev_err);
     cudaFree(c->nonfinite);
@@ -1200,6 +1216,59 @@ empso_status empso_set_levels(empso_ctx *ctx, int32_t grid_id, int32_t n_levels,
     return grid_changed(ctx, grid_id);
 }
 
+namespace {
+
+// A buffer for `graph`, which is being captured (memory nodes in its place would
+// bar the graph from being cloned or used as a child).
+cudaError_t graph_buffer(const std::shared_ptr<GraphBuffers> &from, cudaGraph_t graph, size_t bytes, void **out)
+{
+    size_t k = 0;
+    {
+        std::lock_guard<std::mutex> lock(from->mu);
+        auto &all = from->all;
+        while (k < all.size() && (all[k].taken || all[k].bytes < bytes)) ++k;
+        if (k == all.size()) {
+            // (allowed in this thread's capture once its mode is relaxed: nothing waits)
+            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+            cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
+            if (e != cudaSuccess) return e;
+            void *p = nullptr;
+            e = cudaMalloc(&p, bytes);
+            const cudaError_t back = cudaThreadExchangeStreamCaptureMode(&mode);
+            if (e != cudaSuccess) return e;
+            all.push_back({p, bytes, false});
+            if (back != cudaSuccess) return back;
+        }
+        all[k].taken = true;
+        *out = all[k].p;
+    }
+    // given back when the graph and all that was made from it are gone
+    struct Lease {
+        std::shared_ptr<GraphBuffers> from;
+        size_t k;
+    };
+    const auto give_back = [](void *p) {
+        Lease *l = static_cast<Lease *>(p);
+        {
+            std::lock_guard<std::mutex> lock(l->from->mu);
+            l->from->all[l->k].taken = false;
+        }
+        delete l;
+    };
+    Lease *lease = new Lease{from, k};
+    cudaUserObject_t object;
+    cudaError_t e = cudaUserObjectCreate(&object, lease, give_back, 1, cudaUserObjectNoDestructorSync);
+    if (e != cudaSuccess) {
+        give_back(lease);
+        return e;
+    }
+    e = cudaGraphRetainUserObject(graph, object, 1, cudaGraphUserObjectMove);
+    if (e != cudaSuccess) cudaUserObjectRelease(object);
+    return e;
+}
+
+}  // namespace
+
 empso_status empso_lowpass(empso_ctx *ctx, const float *in, int32_t S, int32_t nt_in, int32_t nrec,
                            double dt_in, float *out, int32_t nt_out, double dt_out, double f_cut,
                            double half_width, void *stream)
@@ -1219,6 +1288,16 @@ empso_status empso_lowpass(empso_ctx *ctx, const float *in, int32_t S, int32_t n
                                             "(half_width / dt_in too large)");
     cudaStream_t st = (cudaStream_t)stream;
     const size_t need = lowpass_ws_floats(S, nrec, nt_out, dt_in, dt_out, half_width, ctx->sm_count);
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    cudaGraph_t graph = nullptr;
+    CK(ctx, cudaStreamGetCaptureInfo(st, &capture, nullptr, &graph));
+    if (capture == cudaStreamCaptureStatusActive) {
+        void *held = nullptr;
+        CK(ctx, graph_buffer(ctx->lp_graphs, graph, sizeof(float) * need, &held));
+        CK(ctx, launch_lowpass(in, S, nt_in, nrec, dt_in, out, nt_out, dt_out, f_cut, half_width, (float *)held, need,
+                               ctx->sm_count, st));
+        return EMPSO_OK;
+    }
     unsigned long long id = 0;
     CK(ctx, cudaStreamGetId(st, &id));
     std::lock_guard<std::mutex> lock(ctx->lp_mu);
@@ -1232,7 +1311,7 @@ empso_status empso_lowpass(empso_ctx *ctx, const float *in, int32_t S, int32_t n
         return EMPSO_OK;
     }
     // from the context's own pool in stream order, so that calls on several streams
-    // do not share it and a capture owns its own
+    // do not share it
     if (!ctx->pool) {
         cudaMemPoolProps props = {};
         props.allocType = cudaMemAllocationTypePinned;

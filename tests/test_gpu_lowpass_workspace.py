@@ -1,5 +1,7 @@
 """The low-pass's workspace: a context's first call finds it made, calls on other
-streams than the first one's take memory of their own."""
+streams than the first one's take memory of their own, a captured call leaves a
+graph that may be cloned and used as a child."""
+import ctypes
 import time
 
 import numpy as np
@@ -64,4 +66,63 @@ def test_streams_do_not_share_a_workspace():
         torch.cuda.synchronize()
         for r, (_, out) in zip(ref, calls):
             assert np.array_equal(out.cpu().numpy(), r)
+    ctx.close()
+
+
+@pytest.mark.parametrize("big", [False, True])
+def test_captured_call_in_clones_and_children(big):
+    """A captured call replayed from the graph, from a clone after the graph is
+    destroyed and from a child of another graph, with direct calls and further
+    captures in between: the bits of direct calls."""
+    rt = ctypes.CDLL("libcudart.so.13")
+    V = ctypes.c_void_p
+
+    def ok(rc):
+        assert rc == 0, rc
+
+    ctx = _ctx()
+    args, out = _call(2, 8000, 461, 8000, 0.5, 4) if big else _call(seed=4)
+    other, _ = _call(2, 3000, 100, 3000, 0.4, 5)
+    x = args[0]
+    st = torch.cuda.Stream()
+
+    def capture(a):
+        graph = V()
+        ok(rt.cudaStreamBeginCapture(V(st.cuda_stream), 0))
+        with torch.cuda.stream(st):
+            ctx.lowpass(*a)
+        ok(rt.cudaStreamEndCapture(V(st.cuda_stream), ctypes.byref(graph)))
+        return graph
+
+    def direct(a, o):
+        o.zero_()
+        ctx.lowpass(*a)
+        torch.cuda.synchronize()
+        return o.cpu().numpy().copy()
+
+    direct(args, out)                       # the kernels are loaded
+    graph = capture(args)
+    clone, parent, node = V(), V(), V()
+    ok(rt.cudaGraphClone(ctypes.byref(clone), graph))
+    ok(rt.cudaGraphCreate(ctypes.byref(parent), 0))
+    ok(rt.cudaGraphAddChildGraphNode(ctypes.byref(node), parent, None, ctypes.c_size_t(0), graph))
+    execs = []
+    for g in (graph, clone, parent):
+        e = V()
+        ok(rt.cudaGraphInstantiate(ctypes.byref(e), g, ctypes.c_ulonglong(0)))
+        ok(rt.cudaGraphDestroy(g))
+        execs.append(e)
+    for k in range(4):
+        x.copy_(torch.randn_like(x))
+        want = direct(args, out)
+        ok(rt.cudaGraphDestroy(capture(other)))          # another table, taken and given back
+        direct(other, other[2])
+        for e in execs:
+            out.zero_()
+            torch.cuda.synchronize()
+            ok(rt.cudaGraphLaunch(e, V(st.cuda_stream)))
+            torch.cuda.synchronize()
+            assert np.array_equal(out.cpu().numpy(), want)
+    for e in execs:
+        ok(rt.cudaGraphExecDestroy(e))
     ctx.close()
