@@ -543,12 +543,16 @@ inline bool group_wide(const GridDev *const *grids, int n_grids)
 // Instances in flight and CTAs per instance: the split of the co-resident CTAs
 // with the least estimated time, rounds of instances x rows a thread sweeps
 // (plus RUN_EXTRA rows' worth for the window it loads first and the step
-// barrier), with at most `by_l2` instances in flight; `fixed` > 0: so many CTAs
-// per instance
+// barrier, of which RUN_BARRIER for the barrier, which one CTA does without), with
+// at most `by_l2` instances in flight; `fixed` > 0: so many CTAs per instance.  The
+// barrier is 1.2 us a step on a GPU of few groups and 1.8 on one of many, a row 0.24:
+// order 8, 103 steps, 1 and 64 models of 21 x 21 + 4 cells 347 and 403 us on groups
+// of 2 CTAs, 258 and 263 on one CTA each; 41 x 31 + 8 cells 366 and 453, 351 and 363;
+// 61 x 41 + 10 cells 402 and 495 on 8 and 4 CTAs, 474 and 504.
 inline WaveSplit group_split(const GridDev *const *grids, int n_grids, int ctas, long long n_inst, long long by_l2,
                              int fixed = 0)
 {
-    constexpr int RUN_EXTRA = 10;
+    constexpr int RUN_EXTRA = 10, RUN_BARRIER = 6;
     WaveSplit best{};
     best.wide = group_wide(grids, n_grids);
     const long long most = std::max<long long>(1, std::min<long long>({n_inst, by_l2, (long long)ctas}));
@@ -558,23 +562,23 @@ inline WaveSplit group_split(const GridDev *const *grids, int n_grids, int ctas,
         best.flight = (int)std::min<long long>(most, ctas / best.group);
         return best;
     }
-    for (long long f = 1; f <= most && ctas > 0; ++f) {
-        const int n = (int)(ctas / f);
-        long long rows = 0;
-        int used = 1;                        // CTAs that have a run to sweep
-        for (int i = 0; i < n_grids; ++i) {
-            const GridDev &g = *grids[i];
-            const int nth = n * WAVE_THREADS, nseg = std::max(1, std::min(g.NZ, nth / g.NQ));
-            rows = std::max<long long>(rows, (long long)((g.NZ + nseg - 1) / nseg) * ((g.NQ * nseg + nth - 1) / nth));
-            used = std::max(used, std::min(n, (g.NQ * nseg + WAVE_THREADS - 1) / WAVE_THREADS));
+    for (long long f = 1; f <= most && ctas > 0; ++f)
+        for (const int n : {(int)(ctas / f), 1}) {       // all the CTAs, or one without a barrier
+            long long rows = 0;
+            int used = 1;                                // CTAs that have a run to sweep
+            for (int i = 0; i < n_grids; ++i) {
+                const GridDev &g = *grids[i];
+                const int nth = n * WAVE_THREADS, nseg = std::max(1, std::min(g.NZ, nth / g.NQ));
+                rows = std::max<long long>(rows, (long long)((g.NZ + nseg - 1) / nseg) * ((g.NQ * nseg + nth - 1) / nth));
+                used = std::max(used, std::min(n, (g.NQ * nseg + WAVE_THREADS - 1) / WAVE_THREADS));
+            }
+            const double c = (double)((n_inst + f - 1) / f) * (double)(rows + RUN_EXTRA - (used == 1 ? RUN_BARRIER : 0));
+            if (best.group == 0 || c < cost) {
+                cost = c;
+                best.flight = (int)f;
+                best.group = used;
+            }
         }
-        const double c = (double)((n_inst + f - 1) / f) * (double)(rows + RUN_EXTRA);
-        if (best.group == 0 || c < cost) {
-            cost = c;
-            best.flight = (int)f;
-            best.group = used;
-        }
-    }
     return best;
 }
 
