@@ -1287,7 +1287,12 @@ empso_status empso_lowpass(empso_ctx *ctx, const float *in, int32_t S, int32_t n
         return fail(ctx, EMPSO_UNSUPPORTED, "filter window too long for shared memory "
                                             "(half_width / dt_in too large)");
     cudaStream_t st = (cudaStream_t)stream;
-    const size_t need = lowpass_ws_floats(S, nrec, nt_out, dt_in, dt_out, half_width, ctx->sm_count);
+    const size_t need = lowpass_ws_floats(S, nt_in, nrec, nt_out, dt_in, dt_out, half_width, ctx->sm_count);
+    if (need == 0) {
+        CK(ctx, launch_lowpass(in, S, nt_in, nrec, dt_in, out, nt_out, dt_out, f_cut, half_width, nullptr, 0, ctx->sm_count,
+                               st));
+        return EMPSO_OK;
+    }
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     cudaGraph_t graph = nullptr;
     CK(ctx, cudaStreamGetCaptureInfo(st, &capture, nullptr, &graph));

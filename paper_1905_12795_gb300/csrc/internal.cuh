@@ -151,7 +151,7 @@ cudaError_t launch_fwi_dots(const float *a, const float *b, const float *c, cons
 
 // Band-limited resampling of traces (filter.cu).
 bool lowpass_supported(double dt_in, double dt_out, double W, size_t limit);
-size_t lowpass_ws_floats(int S, int nrec, int nt_out, double dt_in, double dt_out, double W, int sms);
+size_t lowpass_ws_floats(int S, int nt_in, int nrec, int nt_out, double dt_in, double dt_out, double W, int sms);
 cudaError_t launch_lowpass(const float *in, int S, int nt_in, int nrec, double dt_in, float *out,
                            int nt_out, double dt_out, double fc, double W, float *ws, size_t ws_floats, int sms,
                            cudaStream_t st);
