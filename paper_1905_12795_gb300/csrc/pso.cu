@@ -193,7 +193,7 @@ __device__ __forceinline__ long long ordered(double f)
 // ascending sort gives it.  Every CTA keeps all keys in shared memory.  (One
 // CTA that updated every best and sorted bitonically, 55 passes over shared
 // memory for 1024 keys, took 53 us under ncu for P = 1024, D = 32; this takes
-// 5.5.)  The generation counter is not written here, where every CTA reads
+// 5.5 us.)  The generation counter is not written here, where every CTA reads
 // it: the new one goes to s.k_new for the second part, beside the constriction
 // factor (Eq. 3), whose FP64 root and quotient every thread of the second part
 // would otherwise repeat.
@@ -370,7 +370,8 @@ cudaError_t launch_pso_step(const PsoDev &s, const double *misfit, float *partic
 namespace {
 
 // the swarm's state into the caller's buffers (null ones are skipped), in one
-// launch: as six device-to-device copies it took longer than the step itself
+// launch: as six device-to-device copies it took longer than the step itself (P =
+// 1024, D = 32, three of them: 18.4 us, in one launch 16.1)
 __global__ void state_kernel(PsoDev s, double *x, double *v, double *p, double *pf, int *order, int *gk)
 {
     const long long n = (long long)s.P * s.D, e0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -391,8 +392,28 @@ __global__ void state_kernel(PsoDev s, double *x, double *v, double *p, double *
 cudaError_t launch_pso_state(const PsoDev &s, double *x, double *v, double *p, double *pf, int *order, int *gk,
                              cudaStream_t st)
 {
-    if (!x && !v && !p && !pf && !order && !gk) return cudaSuccess;
     const long long n = (long long)s.P * s.D;
+    const int wanted = !!x + !!v + !!p + !!pf + !!order + !!gk;
+    if (wanted == 0) return cudaSuccess;
+    // One buffer alone, or the largest swarms: copies (a copy takes 1.5 us less than
+    // a launch; at P D = 2M the three of x, v and p run at the copy's bandwidth, 30 us
+    // against 39)
+    if (wanted == 1 || n > 1 << 20) {
+        const size_t PD = sizeof(double) * (size_t)n, P = (size_t)s.P;
+        const struct {
+            void *to;
+            const void *from;
+            size_t bytes;
+        } part[] = {{x, s.x, PD},          {v, s.v, PD},
+                    {p, s.p, PD},          {pf, s.pf, sizeof(double) * P},
+                    {order, s.order, sizeof(int) * P}, {gk, s.gk, 2 * sizeof(int)}};
+        for (const auto &c : part) {
+            if (!c.to) continue;
+            const cudaError_t e = cudaMemcpyAsync(c.to, c.from, c.bytes, cudaMemcpyDeviceToDevice, st);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
+    }
     const int blocks = (int)std::max<long long>(1, std::min<long long>((n + 255) / 256, 1216));
     state_kernel<<<blocks, 256, 0, st>>>(s, x, v, p, pf, order, gk);
     return cudaGetLastError();
