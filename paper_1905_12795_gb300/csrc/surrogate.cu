@@ -535,7 +535,10 @@ __global__ void __launch_bounds__(TC_THREADS) jobs_tc_kernel(const Jobs j, int *
     vector_job(j, b);
 }
 
-__global__ void __launch_bounds__(TC_THREADS) jobs_vector_kernel(const Jobs j) { vector_job(j, blockIdx.x); }
+// (1024 threads: a column sum's threads wait for loads; a gradient over 2000 rows on
+// mma.sync, K = 32, H = 256, took 468 us with 256 of them, 424 with 1024)
+constexpr int VEC_THREADS = 1024;
+__global__ void __launch_bounds__(VEC_THREADS) jobs_vector_kernel(const Jobs j) { vector_job(j, blockIdx.x); }
 
 // the jobs on the context's backend: one launch on tcgen05, else one per product
 cudaError_t run_jobs(const SurDev &s, const Jobs &j, cudaStream_t st)
@@ -551,7 +554,7 @@ cudaError_t run_jobs(const SurDev &s, const Jobs &j, cudaStream_t st)
         const Gemm &g = j.g[i];
         gemm_bf16_kernel<<<dim3((g.N + GBN - 1) / GBN, (g.M + GBM - 1) / GBM), 128, 0, st>>>(g);
     }
-    if (vb) jobs_vector_kernel<<<vb, TC_THREADS, 0, st>>>(j);
+    if (vb) jobs_vector_kernel<<<vb, VEC_THREADS, 0, st>>>(j);
     return cudaGetLastError();
 }
 
