@@ -475,11 +475,13 @@ empso_status empso_level_bounds(int32_t n_levels, const float *level_z,
  * another dt_out it also moves the traces onto that time axis (e.g. data
  * recorded on a fine grid onto the inversion grid's steps).  The transition
  * band is about 3 / half_width Hz wide.  in and out must not overlap.
- * Workspace: 8 MB made with the context serve the first stream that filters;
- * larger tables of taps (up to 64 MB) and other streams take stream-ordered
- * memory of the context's.  A captured call's table stays with the graph, its
- * clones and instantiations; the context outlives their launches.  Errors: INVALID_ARG, UNSUPPORTED (window of more
- * than the shared memory holds: half_width / dt_in too large), OOM. */
+ * Workspace: a table of taps (none for a few taps of short windows).  8 MB
+ * made with the context serve the first stream that filters; larger tables
+ * (up to 64 MB) and other streams take stream-ordered memory of the context's.
+ * A captured call's table stays with the graph, its clones and instantiations;
+ * the context outlives their launches.  Errors: INVALID_ARG, UNSUPPORTED
+ * (window of more than the shared memory holds: half_width / dt_in too large),
+ * OOM. */
 empso_status empso_lowpass(empso_ctx *ctx, const float *in, int32_t S, int32_t nt_in,
                            int32_t nrec, double dt_in, float *out, int32_t nt_out,
                            double dt_out, double f_cut, double half_width, void *stream);
@@ -497,12 +499,13 @@ empso_status empso_lowpass(empso_ctx *ctx, const float *in, int32_t S, int32_t n
  * in time accumulating sum_k mu^k f (L u^{k-1} + s^{k-1}), folded from the
  * damping pad onto the edge nodes and chained through a = v^2 dt^2.  The
  * forward pass runs on the on-chip kernel (history streamed out) when the
- * kernel selection is EMPSO_KERNEL_AUTO or EMPSO_KERNEL_RESIDENT and the grid
+ * order is 8 or less, the kernel selection is EMPSO_KERNEL_AUTO or EMPSO_KERNEL_RESIDENT and the grid
  * fits a cluster (RESIDENT: else UNSUPPORTED); else on the L2 cluster kernel
  * (also streaming the history out) when the selection is EMPSO_KERNEL_AUTO or
  * EMPSO_KERNEL_CLUSTER_L2 and the grid fits it (CLUSTER_L2: else
  * UNSUPPORTED); otherwise (EMPSO_KERNEL_STREAMING) as one launch per time
- * step.  All agree to FP32 rounding.
+ * step.  Order 16 runs on the plain streaming kernel, in one launch, whichever
+ * of AUTO and STREAMING is selected.  All agree to FP32 rounding.
  * misfit: device [M] doubles or NULL; grad: device [M][nz][nx].  d_obs as
  * for eval_models.  Synchronises `stream` once (instance table upload).
  * Errors: INVALID_ARG, OOM (history does not fit), UNSUPPORTED, CUDA_ERROR. */
@@ -510,13 +513,15 @@ empso_status empso_gradient(empso_ctx *ctx, const float *vel, int32_t M,
                             const empso_shot *shots, int32_t S, const float *d_obs,
                             double *misfit, float *grad, void *stream);
 
-/* Chains of the gradient's backward pass: its (model, shot) instances are
- * independent, so they run as n chains (1..8) of consecutive instances on
- * separate streams inside the captured graph, one chain's memory waits and
- * launch gaps overlapping another's work; 0 (default): 4 chains from 16
- * instances up, else 1 (measured on the 461 x 151 grid: 16 shots 35.6 ->
- * 33.3 ms with 4 chains, 4 shots 15.7 -> 18.1 ms).  Results do not depend on
- * n (each instance's arithmetic is the same).  A cluster size set by
+/* Chains of the gradient's backward pass where it runs step by step: more
+ * instances than one round of the persistent pass holds at orders 2 to 8, or
+ * a grid it does not hold.  The (model, shot) instances are independent, so
+ * they run as n chains (1..8) of consecutive instances on separate streams
+ * inside the captured graph, one chain's memory waits and launch gaps
+ * overlapping another's work; 0 (default): 4 chains from 16 instances up, else
+ * 1 (32 shots on the 461 x 151 grid: 52.9 -> 44.7 ms with 4 chains).  The
+ * persistent pass has no chains: there the value is kept and has no effect.
+ * Results do not depend on n (each instance's arithmetic is the same).  A cluster size set by
  * empso_set_cluster also applies to the gradient's on-chip forward pass.
  * An engineering choice of this library (the paper has no such parameter).
  * Errors: INVALID_ARG outside 0..8. */

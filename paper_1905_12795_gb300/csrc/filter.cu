@@ -7,7 +7,7 @@
 // records starting at t = 0 and zero outside them.  With dt_out = dt_in it is
 // a zero-phase low-pass.
 //
-// Two kernels.  lowpass_taps_kernel writes the taps of each tile of LM output
+// Two kernels (one where few taps are formed: lowpass_narrow_kernel).  lowpass_taps_kernel writes the taps of each tile of LM output
 // times, k-major (taps[tile][k][j], k the input sample from the tile's first
 // one, j the output time), once for all shots and receivers: their FP64
 // arguments run at 1/64 of the FP32 rate, and formed by every (shot, 8 output

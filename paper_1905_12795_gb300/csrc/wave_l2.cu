@@ -39,9 +39,10 @@ WaveFn l2_fn(int R, bool hist, bool wide)
 
 }  // namespace
 
-// What the variant takes: slabs of 8 rows or more when the grid is cut into C of
-// them (C = 1 when the library chooses the split), and shots whose receiver
-// tables (28 bytes a receiver) stay within `limit`
+// What the variant takes: at least 8 padded rows for each of the C SMs of an instance
+// (C = 1 when the library chooses the split), and at most as many receivers a shot as
+// tables of 28 bytes each fill `limit` bytes (about 8300).  A group needs neither;
+// they are what EMPSO_KERNEL_CLUSTER_L2 refuses and the streaming kernels take.
 bool l2_fits(const GridDev &g, int C, int nrec, size_t limit)
 {
     const int rows_c = (g.NZ + C - 1) / C;
