@@ -1504,6 +1504,11 @@ __global__ void __launch_bounds__(GRADS_THREADS, 1) grads_kernel(const GradArgs 
         }
         const int t = a.tiles - 1;                 // the last commit covers every product before it
         if (!mbar_wait_tc(smem_u32(&done[t % GSTAGES]), (t / GSTAGES) & 1)) s_fail = 1;
+        // a wait that gave up may have left its copies in flight: they are waited for
+        // once more (bounded) before the CTA gives its shared memory back
+        if (s_fail)
+            for (int i = max(0, a.tiles - GSTAGES); i < a.tiles; ++i)
+                mbar_wait_tc(smem_u32(&full[i % GSTAGES]), (i / GSTAGES) & 1);
     }
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
