@@ -13,7 +13,7 @@
 // The instance runs on a group of co-resident CTAs (wave_group.cuh), with the
 // update as written above.  One CTA of 512 threads per instance, as before,
 // left an order-16 batch of 16 shots on 16 SMs: 1628 ms for 2014 steps of 16
-// shots on the 921 x 301 grid + 60 cells, 43.1 ms on 16 groups of 19 CTAs (327 G
+// shots on the 921 x 301 grid + 60 cells, 43.0 ms on 16 groups of 19 CTAs (328 G
 // updates/s).  Bound by the issue slots (41 % active with 8 warps per SM: the
 // window's 17 rows leave registers for no more) and the barrier.
 #include "wave_group.cuh"

@@ -8,7 +8,7 @@
 //
 // Measured on the grid above, order 8, 16 shots, 2826 steps: 81.7 ms on
 // thread-block clusters of 10 CTAs of 512 threads with a cluster barrier per
-// step (two rounds of 13 clusters, 243 G updates/s), 44.6 ms on groups (444 G
+// step (two rounds of 13 clusters, 243 G updates/s), 44.7 ms on groups (443 G
 // updates/s); 64 shots, 471 steps: 34.8 and 29.8 ms.
 #include "wave_group.cuh"
 
