@@ -216,11 +216,12 @@ lowpass_kernel(LowpassDev p, int tile0, const float *__restrict__ in, float *__r
 
 // Short windows: one launch, a CTA forms the taps of 8 output times in shared memory
 // and takes them over NARROW_COLS columns, one per thread.  The table's second launch
-// costs more than forming the taps again in every CTA while few are formed: 16 shots x
-// 150 x 461 outputs, 56 input samples each, 28 us against 40 with the table, one shot
-// 22 against 27.  Each output is the sum that lowpass_kernel forms, in its order.
-constexpr int NARROW_SPAN = 128, NARROW_COLS = 256;
-constexpr long long NARROW_TAPS = 1 << 19;
+// costs more than forming the taps again in every CTA while few are formed, up to about
+// a million: 16 shots x 150 x 461 outputs, 56 input samples each, 28 us against 40 with
+// the table; 4 x 250 x 162 outputs of 200 samples (150,000 taps) 28 against 36; 16 x 400
+// x 461 of 160 (1.9 million) 60 against 54.  Each output is the sum that lowpass_kernel forms, in its order.
+constexpr int NARROW_SPAN = 256, NARROW_COLS = 256;
+constexpr long long NARROW_TAPS = 1 << 20;
 __global__ void __launch_bounds__(NARROW_COLS)
 lowpass_narrow_kernel(LowpassDev p, float scale, const float *__restrict__ in, float *__restrict__ out)
 {

@@ -9,10 +9,10 @@ from paper_1905_12795_gb300 import synth
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
-SPAN, COLS, TAPS = 128, 256, 1 << 19       # the rule's limits
+SPAN, COLS, TAPS = 256, 256, 1 << 20       # the rule's limits
 
 
-@pytest.mark.parametrize("nt_in,nrec,ratio,half", [(1, 1, 1.0, 0.5), (50, 40, 0.5, 1.0), (128, 257, 1.0, 2.0),
+@pytest.mark.parametrize("nt_in,nrec,ratio,half", [(7, 3, 1.0, 0.5), (50, 40, 0.5, 1.0), (256, 257, 1.0, 2.0),
                                                    (300, 101, 3.7, 0.02), (300, 1, 10.0, 0.02), (1001, 7, 2.0, 0.05)])
 def test_narrow_equals_table(nt_in, nrec, ratio, half):
     from paper_1905_12795_gb300 import binding as B
