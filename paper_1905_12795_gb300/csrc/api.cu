@@ -116,6 +116,16 @@ struct empso_ctx {
     size_t smem_optin = 0;          // max dynamic shared memory per block
     int forced_C = 0;               // 0: choose the cluster size, else use this one
     int forced_rows = 0;            // on-chip kernel: 0 choose the rows per thread, else use this many
+    // on-chip shapes already planned for one grid, by grid, instances and receivers: they
+    // depend on nothing else, and to plan one takes the host some 15 us (one shot of 61 x
+    // 201, order 2: 235 us with the busy-SM rule alone in every call, 243 with the
+    // estimates of some hundred shapes, 224 once planned)
+    struct ResidentShape {
+        int C, rows, threads, nc;
+        size_t sm;
+        std::vector<char> pair;
+    };
+    std::map<std::tuple<int, long long, int>, ResidentShape> res_shapes;
     int last_path = 0;              // 1 streaming, 2 resident, 3 bulk-copy streaming (last launch)
     int last_C = 0;
     int last_rows = 0;              // on-chip launch: rows per thread
@@ -551,21 +561,24 @@ empso_status plan_batch(empso_ctx *ctx, const Models &mod, const empso_shot *sho
         // with the least estimate when that promises 5 % or more (15 % at order 2,
         // where the estimate is rougher: with 5 % there, 36 batches took 2.6 % less
         // on average, but one shot of 301 x 201 279 -> 295 us and 128 of 461 x 151
-        // 3.49 -> 3.57 ms): the busy-SM rule ignores the rounds of instances, the halo rows and how few
-        // threads a long run leaves a small slab, and over 8 grids x 6 batch
-        // sizes was 23 % from the best shape on average (2.05 times at worst),
-        // the estimate 5 % (1.3 times).  101 x 101, order 4: one shot 384 ->
+        // 3.49 -> 3.57 ms): the busy-SM rule ignores the rounds of instances, the halo
+        // rows and how few threads a long run leaves a small slab.  Over 460 batches that
+        // the estimate was not fitted to (61 to 461 columns, orders 2, 4 and 8) the rule
+        // was 31 % from the best shape on average, the estimate 8 %; in 16 of them its
+        // shape was more than 5 % slower than the rule's (at worst 25 %: clusters that
+        // share SMs, which it spreads evenly).  101 x 101, order 4: one shot 384 ->
         // 281 us, 1024 particles 10.99 -> 7.5 ms.
         const bool est = n_grids == 1 && forcedC == 0 && forcedRows == 0;
         double best_us = 0.0, rule_us = 0.0;
-        struct Shape {
-            int C, rows, threads, nc;
-            size_t sm;
-            std::vector<char> pair;
-        } rule{}, least{};
+        empso_ctx::ResidentShape rule{}, least{}, known{};
+        const auto key = std::make_tuple(only, p.n_inst, nrec_max);
+        if (est) {
+            const auto it = ctx->res_shapes.find(key);
+            if (it != ctx->res_shapes.end()) known = it->second;
+        }
         std::vector<int> runs = resident_runs(forcedRows);
         if (est) runs.assign(std::begin(RESIDENT_RUNS_EST), std::end(RESIDENT_RUNS_EST));
-        for (int C = 1; C <= 16; ++C)
+        for (int C = 1; C <= 16 && !known.C; ++C)
             for (const int rows : runs) {
             if (forcedC > 0 && C != forcedC) continue;
             bool ok = true;
@@ -612,7 +625,12 @@ empso_status plan_batch(empso_ctx *ctx, const Models &mod, const empso_shot *sho
                 rule = {C, rows, threads, nc, sm, pair};
             }
         }
-        const Shape &shape = least.C && (!rule.C || best_us * (resR == 1 ? 1.15 : 1.05) < rule_us) ? least : rule;
+        const bool better = least.C && (!rule.C || best_us * (resR == 1 ? 1.15 : 1.05) < rule_us);
+        const auto &shape = known.C ? known : (better ? least : rule);
+        if (est && shape.C && !known.C) {
+            if (ctx->res_shapes.size() >= 256) ctx->res_shapes.clear();
+            ctx->res_shapes[key] = shape;
+        }
         if (shape.C) {
             p.resident = true;
             p.res_pair = shape.pair;
